@@ -440,6 +440,14 @@ int launch(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts
   if (L.drift && (nf || gsum || ghat || prm->ww_lo != 0.0))
     return fail(ctx, WOS_EUNSUPPORTED, "an extra drift (omega) works with the plain solve only");
   const bool fp64 = prm->precision == WOS_FP64;
+  // small FP32 solves spread their walks over the whole chip (walk_sum_kernel adds them up)
+  const bool spread = !fp64 && !nf && !gsum && sum != nullptr && uhat == nullptr && walk_end == nullptr &&
+                      total <= wos::kSpreadItems;
+  if (spread) {
+    L.item_acc = ctx->spread;
+    L.item_iters = reinterpret_cast<uint32_t*>(ctx->spread + wos::kSpreadItems);
+    L.point_scale = ctx->spread + 2 * wos::kSpreadItems;
+  }
   const int variant = (gsum || ghat) ? wos::kJitGrad : (prm->ww_lo != 0.0 ? wos::kJitWindow : wos::kJitPlain);
   cudaKernel_t spec = nf ? nullptr : prob->jit.kernel[fp64 ? 1 : 0][variant];
   if (spec != nullptr) {
@@ -456,6 +464,7 @@ int launch(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts
     L.problem_bytes = (int)sizeof(DevProblem<float>);
     e = nf ? wos::launch_nf_f32(L, ctx->num_sms, st) : wos::launch_walks_f32(L, ctx->num_sms, st);
   }
+  if (e == cudaSuccess && spread) e = wos::launch_walk_sums(L, L.ww_lo == 0.0 && !L.mesh, st);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "walk kernel launch");
   return WOS_OK;
 }
@@ -499,6 +508,10 @@ int wos_create(wos_ctx** out, int device) {
     delete ctx;
     return WOS_ENOMEM;
   }
+  if (cudaMalloc(&ctx->spread, 3 * wos::kSpreadItems * sizeof(float)) != cudaSuccess) {
+    wos_destroy(ctx);
+    return WOS_ENOMEM;
+  }
   if (cudaMemset(ctx->scratch, 0, kScratchWords * sizeof(unsigned long long)) != cudaSuccess ||
       cudaDeviceSynchronize() != cudaSuccess) {
     wos_destroy(ctx);
@@ -514,6 +527,7 @@ int wos_destroy(wos_ctx* ctx) {
   {
     DeviceGuard g(ctx->device);
     cudaFree(ctx->scratch);
+    if (ctx->spread) cudaFree(ctx->spread);
     for (int k = 0; k < 2; ++k)
       if (ctx->radial_tab[k]) cudaFree(ctx->radial_tab[k]);
     if (ctx->walk_end) cudaFree(ctx->walk_end);

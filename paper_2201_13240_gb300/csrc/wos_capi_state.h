@@ -21,6 +21,8 @@ struct wos_ctx {
   std::string err;
   // scratch: [0] work counter, [8..8+ST_WORDS) default stats, [24..29) sigma-bar reduction
   unsigned long long* scratch = nullptr;
+  // per-walk totals, iterations and per-point factors of small solves (3 * kSpreadItems words)
+  float* spread = nullptr;
   // walks-per-point prefix sums
   int64_t* walk_end = nullptr;
   int64_t walk_end_cap = 0;

@@ -32,6 +32,104 @@ cudaError_t launch_walks_kernel(const WalkLaunch& L, cudaKernel_t kernel, int re
   return cudaLaunchKernel(fn, dim3(grid), dim3(kWalkBlock), args, smem, stream);
 }
 
+// Per-point sums of a small solve from its walks' totals (item_acc, in item order).
+//
+// What bounds it: nothing much (8 bytes per walk, ~25 rounds of a warp per 128 walks); it exists
+// so that the walks of a small solve can run one per lane on the whole chip.  The persistent
+// kernel gives a warp 128 walks, four per lane one after another, so a 2^18-walk solve used
+// 2048 warps of the ~3000 that fit and lasted four walks and the longest one's tail.  Measured:
+// 3,000 points x 64 walks on a mesh 476 -> 266 ms, 32^2 x 256 of the 2D square 494 -> 461 us.
+//
+// The order of the sums is the persistent kernel's: FP32 partial sums per lane, shifted by the
+// lane's first walk of the point, over the walks that lane would have run had one warp taken
+// 128 consecutive walks, each lane that is free claiming the next one (lanes free at the same
+// iteration in lane order, GATHERED: once kDeferLanes lanes are free).  A solve's sums therefore
+// do not depend on which warp ran which walk, and equal those of larger chunks' launches.
+template <bool GATHERED>
+__global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__ acc, const uint32_t* __restrict__ iters,
+                                                       const float* __restrict__ scale, uint32_t total,
+                                                       uint32_t walks, double* sum, double* sumsq,
+                                                       unsigned long long* count) {
+  const uint32_t lane = threadIdx.x & 31, base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kChunkMin;
+  if (base >= total) return;
+  const uint32_t n = min((uint32_t)kChunkMin, total - base);
+  constexpr int Q = (int)kChunkMin / 32;
+  float a[Q];
+  uint32_t it[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const bool in = 32 * q + lane < n;
+    a[q] = in ? acc[base + 32 * q + lane] : 0.0f;
+    it[q] = in ? iters[base + 32 * q + lane] : 0u;
+  }
+  uint32_t p = 0xffffffffu, n_acc = 0;
+  float sh = 0.0f, d1 = 0.0f, d2 = 0.0f;
+  auto flush = [&]() {
+    if (n_acc == 0u) return;
+    const double e0 = (double)scale[p], c = (double)sh, m = (double)n_acc;
+    const double s1 = m * c + (double)d1, s2 = m * c * c + 2.0 * c * (double)d1 + (double)d2;
+    atomicAdd(&sum[p], s1 * e0);
+    atomicAdd(&sumsq[p], s2 * e0 * e0);
+    atomicAdd(&count[p], (unsigned long long)n_acc);
+  };
+  auto add = [&](uint32_t item, float v) {
+    const uint32_t q = item / walks;
+    if (q != p) {
+      flush();
+      p = q;
+      n_acc = 0;
+      sh = v;
+      d1 = d2 = 0.0f;
+    }
+    const float dv = v - sh;
+    d1 += dv;
+    d2 += dv * dv;
+    ++n_acc;
+  };
+  if (lane < n) add(base + lane, a[0]);
+  uint32_t free_at = it[0];  // iteration at which the lane has no walk
+  for (uint32_t next = 32; next < n;) {
+    // the iteration of the next claim
+    uint32_t t = __reduce_min_sync(kFull, free_at);
+    if (GATHERED) {
+      uint32_t rest = free_at;
+      for (int got = __popc(__ballot_sync(kFull, rest == t)); got < kDeferLanes;) {
+        if (rest == t) rest = 0xffffffffu;
+        t = __reduce_min_sync(kFull, rest);
+        got += __popc(__ballot_sync(kFull, rest == t));
+      }
+    }
+    const unsigned claim = __ballot_sync(kFull, free_at <= t);
+    const uint32_t j = next + __popc(claim & ((1u << lane) - 1u));
+    float v = 0.0f;
+    uint32_t k = 0;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const float vq = __shfl_sync(kFull, a[q], (int)(j & 31u));
+      const uint32_t kq = __shfl_sync(kFull, it[q], (int)(j & 31u));
+      if ((j >> 5) == (uint32_t)q) {
+        v = vq;
+        k = kq;
+      }
+    }
+    if ((claim >> lane & 1u) && j < n) {
+      add(base + j, v);
+      free_at = t + k;
+    }
+    next += __popc(claim);
+  }
+  flush();
+}
+
+cudaError_t launch_walk_sums(const WalkLaunch& L, bool gathered, cudaStream_t stream) {
+  const uint32_t total = (uint32_t)L.total_items;
+  const uint32_t blocks = (total + 4 * (uint32_t)kChunkMin - 1) / (4 * (uint32_t)kChunkMin);
+  auto* kernel = gathered ? walk_sum_kernel<true> : walk_sum_kernel<false>;
+  kernel<<<blocks, 128, 0, stream>>>(L.item_acc, L.item_iters, L.point_scale, total, (uint32_t)L.walks_uniform, L.sum,
+                                     L.sumsq, L.count);
+  return cudaGetLastError();
+}
+
 int walk_blocks_per_sm_f32(int dim) {
   return dim == 2 ? blocks_per_sm_t<2, float>() : blocks_per_sm_t<3, float>();
 }

@@ -205,6 +205,10 @@ __global__ void __launch_bounds__(kWalkBlock,
   uint64_t chunk = total / ((uint64_t)gridDim.x * (kWalkBlock / 32) * kChunksPerWarp);
   chunk = (chunk < kChunkMin) ? kChunkMin : (chunk > kChunkMax ? kChunkMax : chunk & ~31ull);
   if (L.chunk != 0u) chunk = L.chunk;  // a schedule's choice (a multiple of 32, checked by the host)
+  // small solves: one walk per lane and claim, so that the walks of a launch that does not
+  // fill the chip run side by side; their sums are left to walk_sum_kernel
+  const bool spread = sizeof(R) == 4 && !BATCHED && !GRAD && L.item_acc != nullptr;
+  if (spread) chunk = 32;
   uint64_t chunk_next = 0, chunk_end = 0;
   const uint64_t magic = (L.walks_uniform > 0) ? ~0ull / (uint64_t)L.walks_uniform : 0ull;
   bool exhausted = false;
@@ -250,7 +254,11 @@ __global__ void __launch_bounds__(kWalkBlock,
 #pragma unroll
       for (int i = 0; i < DIM; ++i) gv[i] = (s.k == 0) ? R(NAN) : s.acc * (s.gb[i] - ggam[i]) + s.gc[i];
     }
-    if (accumulate && s.p != acc_p) {
+    if (spread) {
+      L.item_acc[s.item] = (float)s.acc;
+      L.item_iters[s.item] = WW ? s.steps_walk + s.next_bid : s.k + 1u;  // steps and branch ends
+      if (s.w == (uint32_t)L.walk_offset) L.point_scale[s.p] = (float)point_factor<DIM, R>(L, Pw, s.p);
+    } else if (accumulate && s.p != acc_p) {
       if (acc_p != kNoPoint) {
         double e0 = point_factor<DIM, R>(L, BATCHED ? Pall[acc_prob] : *Pshared, acc_p);
         if (!GRAD) {
