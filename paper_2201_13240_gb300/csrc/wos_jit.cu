@@ -242,6 +242,21 @@ std::string kernel_expr(int dim, bool fp64, bool mesh, bool drift, int variant) 
          (drift ? "true" : "false") + ">";
 }
 
+// Resident blocks per SM (the register cap) of the plain walk kernel.  Closed-form fields: 3D 6
+// (80 registers; 7 blocks at 72 registers measured 0.6 % slower, 8 at 64 registers 5 % slower),
+// 2D 8 (64 registers), neither spills.  Cubic B-spline fields keep the support's weights, indices
+// and taps of 4^dim nodes live: at those caps 5-6 % of the executed instructions were spills.
+// Measured with alpha a B-spline, blocks per SM 3 / 4 / 5 / 6 / 7: 3D (4096 points x 512 walks,
+// 16^3 and 33^3 grids) 4.27 / 4.19 / 4.67 / 5.48 / 5.90 and 5.98 / 6.19 / 6.66 / 7.61 / 8.06 ms;
+// 2D (49^2 grids, 4096 x 1024) 3.32 / 3.06 / 3.01 / 3.15 / 3.25 ms and at 8 blocks 3.42 ms; a
+// batch of 192 2D problems 117.6 / 107.9 / 106.5 / 110.0 / 111.5 ms and at 8 blocks 117.4 ms.
+int min_blocks(const DevProblem<double>& P, bool batch) {
+  const DevField<double>* fields[6] = {&P.alpha, &P.phi, &P.sigma, &P.f, &P.g, &P.um};
+  for (const DevField<double>* f : fields)
+    if (f->kind == F_GRID_BSPLINE) return P.dim == 3 ? 4 : 5;
+  return P.dim == 3 ? (batch ? 7 : 6) : 8;
+}
+
 }  // namespace
 
 std::string jit_source(const DevProblem<double>& P) {
@@ -259,9 +274,7 @@ std::string jit_source(const DevProblem<double>& P) {
     for (int i = 0; i < 16; ++i) s += (i ? ", " : "") + lit(P.dom[i]);
     s += "}\n";
   }
-  // resident blocks per SM: 3D 6 (80 registers; 7 blocks at 72 registers measured 0.6 %
-  // slower, 8 at 64 registers 5 % slower), 2D 8 (64 registers), neither spills
-  s += (dim == 3) ? "#define WOS_WALK_MIN_BLOCKS 6\n" : "#define WOS_WALK_MIN_BLOCKS 8\n";
+  s += "#define WOS_WALK_MIN_BLOCKS " + std::to_string(min_blocks(P, false)) + "\n";
   s += "#include \"wos_walk_impl.cuh\"\n#include \"wos_adjoint_impl.cuh\"\n\nnamespace wos {\n\n";
   s += "template <int DIM, typename R>\n";
   s += "__device__ __forceinline__ FieldVal<R> jit_field(const DevProblem<R>& P, int id, R x0, R x1, R x2, "
@@ -305,7 +318,7 @@ std::string jit_source_batch(const BatchJitInfo& info) {
        "D): fields shared by every problem are generated code, the others are interpreted\n";
   s += "#define WOS_JIT_FIELDS 1\n";
   s += "#define WOS_JIT_F_KIND " + std::to_string(P.f.kind) + "\n";
-  s += (dim == 3) ? "#define WOS_WALK_MIN_BLOCKS 7\n" : "#define WOS_WALK_MIN_BLOCKS 8\n";
+  s += "#define WOS_WALK_MIN_BLOCKS " + std::to_string(min_blocks(P, true)) + "\n";
   s += "#include \"wos_walk_impl.cuh\"\n\nnamespace wos {\n\n";
   s += "template <int DIM, typename R>\n";
   s += "__device__ __forceinline__ FieldVal<R> jit_field(const DevProblem<R>& P, int id, R x0, R x1, R x2, "
