@@ -21,7 +21,7 @@ struct wos_ctx {
   std::string err;
   // scratch: [0] work counter, [8..8+ST_WORDS) default stats, [24..29) sigma-bar reduction
   unsigned long long* scratch = nullptr;
-  // per-walk totals, iterations and per-point factors of small solves (3 * kSpreadItems words)
+  // per-walk totals, iterations and points and per-point factors of small solves (wos::use_spread)
   float* spread = nullptr;
   // walks-per-point prefix sums
   int64_t* walk_end = nullptr;

@@ -17,6 +17,11 @@ enum {
   ST_MESH_NODES = 6, ST_MESH_TRIS = 7, ST_EXHAUSTED = 8, ST_WORDS = 9
 };
 
+// Largest launch (walks) that takes the per-walk buffers of a small solve (16 MB per context): about
+// ten walks for each lane of the chip; a larger launch keeps every lane busy by itself (1.67e6
+// walks: 1.02 ms either way).
+constexpr uint64_t kSpreadItems = 1ull << 20;
+
 struct WalkLaunch {
   const void* problem;            // DevProblem<R> in device memory
   int problem_bytes;              // sizeof(DevProblem<R>), multiple of 16
@@ -62,10 +67,12 @@ struct WalkLaunch {
   uint32_t chunk;
   int32_t blocks_per_sm;
   int32_t regs_variant;
-  // small solves (null otherwise): the walk kernel writes each walk's U-space total and its
-  // loop iterations here, and walk_sum_kernel adds them up per point (see launch_walk_sums)
-  float* item_acc;                // [total_items]
-  uint32_t* item_iters;           // [total_items]
+  // small solves (null otherwise, and used while the launch has at most kSpreadItems walks): the
+  // walk kernel writes each walk's U-space total, its loop iterations and its point here, and
+  // walk_sum_kernel adds them up per point (see launch_walk_sums)
+  float* item_acc;                // [kSpreadItems]
+  uint32_t* item_iters;           // [kSpreadItems]
+  uint32_t* item_point;           // [kSpreadItems]
   float* point_scale;             // [npts] e^{-gamma(x_0)}
   // Philox round keys of `seed`, set by the launch functions (philox_round_keys): in the
   // kernel's parameter space each round's key is a constant operand of the XOR
@@ -116,13 +123,16 @@ cudaError_t launch_walks_f64(const WalkLaunch& L, int num_sms, cudaStream_t stre
 cudaError_t launch_walks_kernel(const WalkLaunch& L, cudaKernel_t kernel, int real_bytes, int num_sms,
                                 cudaStream_t stream);
 
-// largest launch (walks) that takes the per-walk buffers above (12 MB per context): about ten
-// walks for each lane of the chip; a larger launch keeps every lane busy by itself (1.67e6
-// walks: 1.02 ms either way)
-constexpr uint64_t kSpreadItems = 1ull << 20;
 // adds the walks of a launch with per-walk buffers to L.sum, L.sumsq and L.count; `gathered`:
 // the walk kernel's lanes wait for each other's ends (kDeferLanes)
 cudaError_t launch_walk_sums(const WalkLaunch& L, bool gathered, cudaStream_t stream);
+// per-walk buffers of a context in `buf` (4 * kSpreadItems words) for a launch that may take them
+inline void use_spread(WalkLaunch* L, float* buf) {
+  L->item_acc = buf;
+  L->item_iters = reinterpret_cast<uint32_t*>(buf + kSpreadItems);
+  L->item_point = reinterpret_cast<uint32_t*>(buf + 2 * kSpreadItems);
+  L->point_scale = buf + 3 * kSpreadItems;
+}
 
 // next-flight walks (Sec. 5.2)
 cudaError_t launch_nf_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream);

@@ -34,7 +34,7 @@ cudaError_t launch_walks_kernel(const WalkLaunch& L, cudaKernel_t kernel, int re
 
 // Per-point sums of a small solve from its walks' totals (item_acc, in item order).
 //
-// What bounds it: nothing much (8 bytes per walk, ~25 rounds of a warp per 128 walks); it exists
+// What bounds it: nothing much (12 bytes per walk, ~25 rounds of a warp per 128 walks); it exists
 // so that the walks of a small solve can run one per lane on the whole chip.  The persistent
 // kernel gives a warp 128 walks, four per lane one after another, so a 2^18-walk solve used
 // 2048 warps of the ~3000 that fit and lasted four walks and the longest one's tail.  Measured:
@@ -47,9 +47,13 @@ cudaError_t launch_walks_kernel(const WalkLaunch& L, cudaKernel_t kernel, int re
 // do not depend on which warp ran which walk, and equal those of larger chunks' launches.
 template <bool GATHERED>
 __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__ acc, const uint32_t* __restrict__ iters,
-                                                       const float* __restrict__ scale, uint32_t total,
-                                                       uint32_t walks, double* sum, double* sumsq,
-                                                       unsigned long long* count) {
+                                                       const uint32_t* __restrict__ point,
+                                                       const float* __restrict__ scale, uint64_t all,
+                                                       const int64_t* walk_end, int64_t npts, double* sum,
+                                                       double* sumsq, unsigned long long* count) {
+  if (walk_end != nullptr) all = (uint64_t)__ldg(&walk_end[npts - 1]);  // per-point walk counts
+  if (all > kSpreadItems) return;  // the walk kernel added these up itself
+  const uint32_t total = (uint32_t)all;
   const uint32_t lane = threadIdx.x & 31, base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kChunkMin;
   if (base >= total) return;
   const uint32_t n = min((uint32_t)kChunkMin, total - base);
@@ -73,7 +77,7 @@ __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__
     atomicAdd(&count[p], (unsigned long long)n_acc);
   };
   auto add = [&](uint32_t item, float v) {
-    const uint32_t q = item / walks;
+    const uint32_t q = point[item];
     if (q != p) {
       flush();
       p = q;
@@ -122,11 +126,11 @@ __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__
 }
 
 cudaError_t launch_walk_sums(const WalkLaunch& L, bool gathered, cudaStream_t stream) {
-  const uint32_t total = (uint32_t)L.total_items;
-  const uint32_t blocks = (total + 4 * (uint32_t)kChunkMin - 1) / (4 * (uint32_t)kChunkMin);
+  const uint64_t most = (L.total_items < kSpreadItems) ? L.total_items : kSpreadItems;
+  const uint64_t blocks = (most + 4 * kChunkMin - 1) / (4 * kChunkMin);
   auto* kernel = gathered ? walk_sum_kernel<true> : walk_sum_kernel<false>;
-  kernel<<<blocks, 128, 0, stream>>>(L.item_acc, L.item_iters, L.point_scale, total, (uint32_t)L.walks_uniform, L.sum,
-                                     L.sumsq, L.count);
+  kernel<<<(unsigned)blocks, 128, 0, stream>>>(L.item_acc, L.item_iters, L.item_point, L.point_scale, L.total_items,
+                                               L.walk_end, L.npts, L.sum, L.sumsq, L.count);
   return cudaGetLastError();
 }
 

@@ -77,9 +77,29 @@ __device__ __forceinline__ double point_factor(const WalkLaunch& L, const DevPro
   return (double)w_exp(-gamma_at<DIM>(P, x0));
 }
 
+// The smallest i in [i, n) whose ends[i] exceeds v (n - 1 if none), given that no earlier one
+// does: steps from i that double until one is passed, then bisection.  A warp's walks are
+// consecutive items, so they lie in the last claim's point or a few after it: one or two loads,
+// where bisecting all points and problems for every walk took ~25 dependent loads (with the
+// prefix kernel's wider passes: 192 2D problems, 5.7e7 walks, 106.5 -> 103.3 ms).
+__device__ __forceinline__ uint32_t first_above(const int64_t* ends, uint32_t i, uint32_t n, uint64_t v) {
+  uint32_t hi = i, step = 1;
+  while (hi < n - 1 && (uint64_t)__ldg(&ends[hi]) <= v) {
+    i = hi + 1;
+    hi = (n - 1 - hi > step) ? hi + step : n - 1;
+    step <<= 1;
+  }
+  while (i < hi) {
+    const uint32_t mid = i + (hi - i) / 2;
+    if ((uint64_t)__ldg(&ends[mid]) > v) hi = mid; else i = mid + 1;
+  }
+  return i;
+}
+
+// cur_p, cur_prob: a point and a problem that begin at or before `item` (the warp's last claim's)
 template <int DIM, typename R, bool BATCHED>
-__device__ __forceinline__ void start_walk(const WalkLaunch& L, uint64_t item, uint64_t magic,
-                                           WalkState<DIM, R>& s) {
+__device__ __forceinline__ void start_walk(const WalkLaunch& L, uint64_t item, uint64_t magic, uint32_t cur_p,
+                                           uint32_t cur_prob, WalkState<DIM, R>& s) {
   uint64_t p, j;
   if (L.walk_end == nullptr) {
     // item / walks_uniform by a multiply-high with magic = floor((2^64 - 1) / walks_uniform):
@@ -93,27 +113,14 @@ __device__ __forceinline__ void start_walk(const WalkLaunch& L, uint64_t item, u
     }
   } else {
     // first point whose inclusive walk prefix exceeds item
-    int64_t lo = 0, hi = L.npts - 1;
-    while (lo < hi) {
-      int64_t mid = (lo + hi) >> 1;
-      if ((uint64_t)__ldg(&L.walk_end[mid]) > item) hi = mid; else lo = mid + 1;
-    }
-    p = (uint64_t)lo;
-    uint64_t begin = (lo > 0) ? (uint64_t)__ldg(&L.walk_end[lo - 1]) : 0ull;
-    j = item - begin;
+    p = first_above(L.walk_end, cur_p, (uint32_t)L.npts, item);
+    j = item - ((p > 0) ? (uint64_t)__ldg(&L.walk_end[p - 1]) : 0ull);
   }
   s.item = item;
   s.p = (uint32_t)p;
   s.prob = 0;
-  if (BATCHED) {
-    // the problem whose point range holds p: last offset <= p
-    int lo = 0, hi = L.nprob - 1;
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if ((uint64_t)__ldg(&L.prob_offsets[mid]) <= p) lo = mid; else hi = mid - 1;
-    }
-    s.prob = (uint32_t)lo;
-  }
+  // the problem whose point range holds p: the first whose range's end exceeds it
+  if (BATCHED) s.prob = first_above(L.prob_offsets + 1, cur_prob, (uint32_t)L.nprob, p);
   s.w = (uint32_t)(L.walk_offset + j);
   s.k = 0;
 #pragma unroll
@@ -207,9 +214,10 @@ __global__ void __launch_bounds__(kWalkBlock,
   if (L.chunk != 0u) chunk = L.chunk;  // a schedule's choice (a multiple of 32, checked by the host)
   // small solves: one walk per lane and claim, so that the walks of a launch that does not
   // fill the chip run side by side; their sums are left to walk_sum_kernel
-  const bool spread = sizeof(R) == 4 && !BATCHED && !GRAD && L.item_acc != nullptr;
+  const bool spread = sizeof(R) == 4 && !GRAD && L.item_acc != nullptr && total <= kSpreadItems;
   if (spread) chunk = 32;
   uint64_t chunk_next = 0, chunk_end = 0;
+  uint32_t cur_p = 0, cur_prob = 0;
   const uint64_t magic = (L.walks_uniform > 0) ? ~0ull / (uint64_t)L.walks_uniform : 0ull;
   bool exhausted = false;
   bool active = false;
@@ -256,6 +264,7 @@ __global__ void __launch_bounds__(kWalkBlock,
     }
     if (spread) {
       L.item_acc[s.item] = (float)s.acc;
+      L.item_point[s.item] = s.p;
       L.item_iters[s.item] = WW ? s.steps_walk + s.next_bid : s.k + 1u;  // steps and branch ends
       if (s.w == (uint32_t)L.walk_offset) L.point_scale[s.p] = (float)point_factor<DIM, R>(L, Pw, s.p);
     } else if (accumulate && s.p != acc_p) {
@@ -356,9 +365,15 @@ __global__ void __launch_bounds__(kWalkBlock,
         uint64_t avail = chunk_end - chunk_next;
         unsigned take = (avail < nneed) ? (unsigned)avail : nneed;
         unsigned rank = __popc(need & lt_mask);
-        if (!active && rank < take) {
-          start_walk<DIM, R, BATCHED>(L, chunk_next + rank, magic, s);
+        const bool claims = !active && rank < take;
+        if (claims) {
+          start_walk<DIM, R, BATCHED>(L, chunk_next + rank, magic, cur_p, cur_prob, s);
           active = true;
+        }
+        if (BATCHED || L.walk_end != nullptr) {  // the last claimed item's point and problem
+          const int last = 31 - __clz(__ballot_sync(kFull, claims));
+          cur_p = __shfl_sync(kFull, s.p, last);
+          if (BATCHED) cur_prob = __shfl_sync(kFull, s.prob, last);
         }
         chunk_next += take;
         need = __ballot_sync(kFull, !active);

@@ -42,3 +42,25 @@ def test_sums_equal_the_walks(kind, npts, walks):
     # at most 4 max u^2
     big = u.abs().max(1).values ** 2 * walks
     assert torch.all((s2 - u.square().sum(1)).abs() <= 8 * tol * big)
+
+
+@pytest.mark.parametrize("most", [1, 3, 200, 5000])
+def test_per_point_counts(most):
+    """Walks per point from 0 up (runs of points without walks among them): counts are exact, and the
+    sums are those of the walks' own estimates (rounding as above, with at most `most` walks of a
+    point in a lane); most = 5000 is above the small-solve limit of 2^20 walks."""
+    import torch
+    ctx = _ctx()
+    prob = ctx.problem(W.square2d_problem())
+    npts = 700
+    pts = torch.from_numpy(W.uniform_in_box(2, npts, 0.02, 0.98, 5)).cuda()
+    rng = np.random.default_rng(most)
+    counts = rng.integers(0, most + 1, npts).astype(np.int32)
+    counts[100:400:1 if most == 1 else 7] = 0
+    counts[-1] = 0
+    (s, s2, n), st = ctx.solve(prob, pts, torch.from_numpy(counts).cuda(), 1e-3, 50.0, seed=7)
+    assert np.array_equal(n.cpu().numpy(), counts) and int(st[1]) == int(counts.sum())
+    u, _, _ = ctx.walk_estimates(prob, pts, most, 1e-3, 50.0, seed=7)
+    u = torch.where(torch.arange(most, device="cuda")[None, :] < torch.from_numpy(counts).cuda()[:, None], u, 0.0)
+    tol = max(128, most) * 2.0 ** -24
+    assert torch.all((s - u.sum(1)).abs() <= tol * u.abs().sum(1))
