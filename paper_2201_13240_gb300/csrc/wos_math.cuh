@@ -140,6 +140,8 @@ WOS_HD void w_sincospi2(double u, double* s, double* c) {
   *c = cos(6.283185307179586476925 * u);
 #endif
 }
+WOS_HD float w_fma(float a, float b, float c) { return fmaf(a, b, c); }
+WOS_HD double w_fma(double a, double b, double c) { return fma(a, b, c); }
 WOS_HD float w_cbrt(float x) { return cbrtf(x); }
 WOS_HD double w_cbrt(double x) { return cbrt(x); }
 WOS_HD float w_expm1(float x) { return expm1f(x); }

@@ -447,6 +447,13 @@ WOS_HD R box_d2(const R* x, const F4& lo, const F4& hi) {
   return dx * dx + dy * dy + dz * dz;
 }
 
+// a . b, its roundings spelled out: the mesh queries give the same bits in whichever kernel they
+// are compiled (left to the compiler, the choice of the product that is rounded varies)
+template <typename R>
+WOS_HD R dot3(const R* a, const R* b) {
+  return w_fma(a[2], b[2], w_fma(a[0], b[0], a[1] * b[1]));
+}
+
 // Closest point of triangle (a, b, c) to p by its Voronoi regions (Ericson,
 // Real-Time Collision Detection, Sec. 5.1.5): barycentric (v, w) of the point.
 template <typename R>
@@ -455,15 +462,12 @@ WOS_HD void tri_closest(const R* p, const float* t, R* v_out, R* w_out, R* d2_ou
   R ab[3] = {R(B.x) - R(A.x), R(B.y) - R(A.y), R(B.z) - R(A.z)};
   R ac[3] = {R(Cc.x) - R(A.x), R(Cc.y) - R(A.y), R(Cc.z) - R(A.z)};
   R ap[3] = {p[0] - R(A.x), p[1] - R(A.y), p[2] - R(A.z)};
-  R d1 = ab[0] * ap[0] + ab[1] * ap[1] + ab[2] * ap[2];
-  R d2 = ac[0] * ap[0] + ac[1] * ap[1] + ac[2] * ap[2];
-  R abab = ab[0] * ab[0] + ab[1] * ab[1] + ab[2] * ab[2];
-  R acac = ac[0] * ac[0] + ac[1] * ac[1] + ac[2] * ac[2];
-  R abac = ab[0] * ac[0] + ab[1] * ac[1] + ab[2] * ac[2];
+  R d1 = dot3(ab, ap), d2 = dot3(ac, ap);
+  R abab = dot3(ab, ab), acac = dot3(ac, ac), abac = dot3(ab, ac);
   R d3 = d1 - abab, d4 = d2 - abac;  // ab.(p-b), ac.(p-b)
   R d5 = d1 - abac, d6 = d2 - acac;  // ab.(p-c), ac.(p-c)
   R v, w;
-  R vc = d1 * d4 - d3 * d2, vb = d5 * d2 - d1 * d6, va = d3 * d6 - d5 * d4;
+  R vc = w_fma(d1, d4, -(d3 * d2)), vb = w_fma(d5, d2, -(d1 * d6)), va = w_fma(d3, d6, -(d5 * d4));
   if (d1 <= R(0) && d2 <= R(0)) { v = R(0); w = R(0); }                       // vertex a
   else if (d3 >= R(0) && d4 <= d3) { v = R(1); w = R(0); }                    // vertex b
   else if (d6 >= R(0) && d5 <= d6) { v = R(0); w = R(1); }                    // vertex c
@@ -477,10 +481,12 @@ WOS_HD void tri_closest(const R* p, const float* t, R* v_out, R* w_out, R* d2_ou
     v = vb * den;
     w = vc * den;
   }
-  R q[3] = {ap[0] - ab[0] * v - ac[0] * w, ap[1] - ab[1] * v - ac[1] * w, ap[2] - ab[2] * v - ac[2] * w};
+  R q[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) q[i] = w_fma(-ac[i], w, w_fma(-ab[i], v, ap[i]));
   *v_out = v;
   *w_out = w;
-  *d2_out = q[0] * q[0] + q[1] * q[1] + q[2] * q[2];
+  *d2_out = dot3(q, q);
 }
 
 template <typename R>
@@ -554,144 +560,276 @@ WOS_HD I4 lds4i(const float* p) {
   return v;
 #endif
 }
+WOS_HD int ld1i(const float* p) {
+#if defined(__CUDA_ARCH__)
+  return __ldg(reinterpret_cast<const int*>(p));
+#else
+  int v;
+  memcpy(&v, p, 4);
+  return v;
+#endif
+}
 template <typename R>
 WOS_HD R box_d2_1(const R* x, float lx, float ly, float lz, float hx, float hy, float hz) {
-  R dx = w_fmax(w_fmax(R(lx) - x[0], x[0] - R(hx)), R(0));
-  R dy = w_fmax(w_fmax(R(ly) - x[1], x[1] - R(hy)), R(0));
-  R dz = w_fmax(w_fmax(R(lz) - x[2], x[2] - R(hz)), R(0));
-  return dx * dx + dy * dy + dz * dz;
+  const R dx = w_fmax(w_fmax(R(lx) - x[0], x[0] - R(hx)), R(0));
+  const R dy = w_fmax(w_fmax(R(ly) - x[1], x[1] - R(hy)), R(0));
+  const R dz = w_fmax(w_fmax(R(lz) - x[2], x[2] - R(hz)), R(0));
+  return w_fma(dz, dz, w_fma(dy, dy, dx * dx));
 }
 
+// One closest-point search as a resumable state: node_step() leaves the current node (sorts its
+// interior children, pushes the farther ones) and visits the next; when a leaf child is within the
+// threshold the caller finds the leaf's nearest triangle (lt .. le - 1) and reports it to
+// leaf_done().  `sub` says which comes next.  The order of the visits and tests is the depth-first
+// order above whoever calls them, so a kernel may run its lanes at different speeds.
+enum MeshSub { MS_NODE = 0, MS_TRI = 1, MS_DONE = 2 };
+template <typename R>
+struct MeshSearch {
+  R best, bv, bw;              // squared distance and barycentrics of the best triangle
+  R tau;
+  R d[4];                      // squared box distances of the current node's children
+  int c[4];                    // their child indices (interior) or first triangles (leaves)
+  int best_t;
+  int node;                    // the node whose children d, c hold
+  int lt, le;                  // leaf under test: next triangle, end
+  int sp;                      // stack entries
+  int sub;                     // MeshSub
+  uint32_t kind;               // bits 0-3 interior children, 4-7 leaf children not yet tested
+  int pass;
+  bool again;
+  uint32_t n_nodes, n_tris;
+
+  WOS_HD void restart(int* sn, R* sd) {
+    again = false;
+    kind = 0;                  // no children to leave: node_step() pops the root
+    sn[0] = 0;
+    sd[0] = R(-1);
+    sp = 1;
+    sub = MS_NODE;
+  }
+  WOS_HD void begin(R bound2, R tau_, int* sn, R* sd) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      d[i] = R(INFINITY);
+      c[i] = 0;
+    }
+    const R slack = (sizeof(R) == 4) ? R(1e-5) : R(1e-12);
+    best = (bound2 < R(INFINITY)) ? w_fma(bound2, R(1) + slack, R(1e-30)) : R(INFINITY);
+    bv = R(0);
+    bw = R(0);
+    best_t = -1;
+    tau = tau_;
+    node = 0;
+    lt = le = 0;
+    pass = 0;
+    n_nodes = n_tris = 0;
+    restart(sn, sd);
+  }
+  // the next untested leaf child within the opening threshold
+  WOS_HD void next_leaf(const DevProblem<R>& P) {
+    sub = MS_NODE;
+    const R thr = tau * best;
+    int at = -1;
+#pragma unroll
+    for (int i = 3; i >= 0; --i)
+      if (((kind >> (4 + i)) & 1u) && d[i] < thr) {
+        at = i;
+        lt = c[i];
+      }
+    if (at < 0) return;
+    kind &= ~((2u << at) - 1u) << 4 | 0xfu;  // this leaf and the ones before it are done
+    const int n = ld1i(P.mesh_nodes + 32 * node + 28 + at);
+    le = lt + n;
+    n_tris += (uint32_t)n;
+    sub = MS_TRI;
+  }
+  // the nearest triangle of the leaf under test (d2 at v, w) is known: on to the next leaf
+  WOS_HD void leaf_done(const DevProblem<R>& P, R d2, R v, R w, int t) {
+    if (d2 < best) {
+      best = d2;
+      best_t = t;
+      bv = v;
+      bw = w;
+    }
+    next_leaf(P);
+  }
+  WOS_HD void node_step(const DevProblem<R>& P, const R* x, int* stk_n, R* stk_d, int sst, const float* top) {
+    const R thr = tau * best;
+    // leave the current node: interior children within the threshold, nearest first
+    R k[4];
+    int e[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      k[i] = (((kind >> i) & 1u) && d[i] < thr) ? d[i] : R(INFINITY);
+      e[i] = c[i];
+    }
+#define WOS_CSWAP(a, b)                                   \
+  if (k[b] < k[a]) {                                      \
+    R tk = k[a]; k[a] = k[b]; k[b] = tk;                  \
+    int tc = e[a]; e[a] = e[b]; e[b] = tc;                \
+  }
+    WOS_CSWAP(0, 1) WOS_CSWAP(2, 3) WOS_CSWAP(0, 2) WOS_CSWAP(1, 3) WOS_CSWAP(1, 2)
+#undef WOS_CSWAP
+    // push the farther ones (farthest first, so the nearer are popped first)
+#pragma unroll
+    for (int i = 3; i >= 1; --i) {
+      if (k[i] < thr) {
+        if (sp < kMeshStack) {
+          stk_n[sp * sst] = e[i];
+          stk_d[sp * sst] = k[i];
+          ++sp;
+        } else {
+          again = true;
+        }
+      }
+    }
+    bool found = k[0] < thr;
+    node = found ? e[0] : node;
+    // else pop the next node still within the threshold of the best triangle
+    while (!found && sp > 0) {
+      --sp;
+      if (stk_d[sp * sst] < thr) {
+        node = stk_n[sp * sst];
+        found = true;
+      }
+    }
+    if (!found) {
+      // the pass ends.  Exact: a pass that found nothing within its bound, or dropped stack
+      // entries, is followed by one from the root with the best so far (or none).  tau < 1: only
+      // a pass that dropped entries is repeated, from the best so far.
+      const bool none = best_t < 0 && !(tau < R(1));
+      if (++pass < 8 && (again || none)) {
+        if (none) best = R(INFINITY);
+        restart(stk_n, stk_d);
+      } else {
+        sub = MS_DONE;
+      }
+      return;
+    }
+    // visit the node
+    F4 lx, ly, lz, hx, hy, hz;
+    I4 ch, cn;
+    if (top != nullptr && node < P.mesh_top) {
+      // one of the tree's top nodes, staged in shared memory by the kernel
+      const float* nd = top + 32 * node;
+      lx = lds4(nd); ly = lds4(nd + 4); lz = lds4(nd + 8);
+      hx = lds4(nd + 12); hy = lds4(nd + 16); hz = lds4(nd + 20);
+      ch = lds4i(nd + 24); cn = lds4i(nd + 28);
+    } else {
+      const float* nd = P.mesh_nodes + 32 * node;
+      lx = ld4(nd); ly = ld4(nd + 4); lz = ld4(nd + 8);
+      hx = ld4(nd + 12); hy = ld4(nd + 16); hz = ld4(nd + 20);
+      ch = ld4i(nd + 24); cn = ld4i(nd + 28);
+    }
+    ++n_nodes;
+    d[0] = box_d2_1(x, lx.x, ly.x, lz.x, hx.x, hy.x, hz.x);
+    d[1] = box_d2_1(x, lx.y, ly.y, lz.y, hx.y, hy.y, hz.y);
+    d[2] = box_d2_1(x, lx.z, ly.z, lz.z, hx.z, hy.z, hz.z);
+    d[3] = box_d2_1(x, lx.w, ly.w, lz.w, hx.w, hy.w, hz.w);
+    c[0] = ch.x; c[1] = ch.y; c[2] = ch.z; c[3] = ch.w;
+    kind = (cn.x == 0 ? 1u : 0u) | (cn.y == 0 ? 2u : 0u) | (cn.z == 0 ? 4u : 0u) | (cn.w == 0 ? 8u : 0u) |
+           (cn.x > 0 ? 16u : 0u) | (cn.y > 0 ? 32u : 0u) | (cn.z > 0 ? 64u : 0u) | (cn.w > 0 ? 128u : 0u);
+    // leaf children within the opening threshold are tested first (they lower best)
+    if (kind >> 4) next_leaf(P);
+  }
+  // the result of a finished search (see mesh_query)
+  WOS_HD MeshHit<R> hit(const DevProblem<R>& P, const R* x, const R* pb, MeshVisits* vis) const {
+    const bool exact = !(tau < R(1));
+    MeshHit<R> h;
+    if (vis != nullptr) {
+      vis->nodes += n_nodes;
+      vis->tris += n_tris;
+    }
+    if (best_t >= 0) {
+      const float* t = P.mesh_tris + 12 * best_t;
+      F4 A = ld4(t), B = ld4(t + 4), Cc = ld4(t + 8);
+      h.x = w_fma(R(Cc.x) - R(A.x), bw, w_fma(R(B.x) - R(A.x), bv, R(A.x)));
+      h.y = w_fma(R(Cc.y) - R(A.y), bw, w_fma(R(B.y) - R(A.y), bv, R(A.y)));
+      h.z = w_fma(R(Cc.z) - R(A.z), bw, w_fma(R(B.z) - R(A.z), bv, R(A.z)));
+      h.d = exact ? w_sqrt(best) : w_sqrt(tau * best);
+    } else if (!exact && best < R(INFINITY)) {
+      // nothing inside the bound: its own boundary point (when known) is the best point
+      h.x = pb ? pb[0] : R(NAN);
+      h.y = pb ? pb[1] : R(NAN);
+      h.z = pb ? pb[2] : R(NAN);
+      h.d = w_sqrt(tau * best);
+    } else {
+      // no boundary point found at all (eight passes of overflowing stacks, or a non-finite
+      // point): counted, and the walk ends here (distance 0, closest point x)
+      if (vis != nullptr) ++vis->exhausted;
+      h.x = x[0];
+      h.y = x[1];
+      h.z = x[2];
+      h.d = R(0);
+    }
+    return h;
+  }
+};
+
+// A whole search by one lane (the kernels whose lanes search in step, and the host).
 template <typename R, bool SMEM>
 WOS_FIELD_FN MeshHit<R> mesh_query(const DevProblem<R>& P, R x0, R x1, R x2, R bound2, int* sn, R* sd,
                                    int stride, R tau = R(1), const R* pb = nullptr, MeshVisits* vis = nullptr,
                                    const float* top = nullptr) {
   const R x[3] = {x0, x1, x2};
-  const float* nodes = P.mesh_nodes;
-  const float* tris = P.mesh_tris;
   int loc_n[SMEM ? 1 : kMeshStack];
   R loc_d[SMEM ? 1 : kMeshStack];
   int* stk_n = SMEM ? sn : loc_n;
   R* stk_d = SMEM ? sd : loc_d;
-  const int sst = SMEM ? stride : 1;
-  const bool exact = !(tau < R(1));
-  R best = R(INFINITY), bv = R(0), bw = R(0);
-  int best_t = -1;
-  const R slack = (sizeof(R) == 4) ? R(1e-5) : R(1e-12);
-  const R start = (bound2 < R(INFINITY)) ? bound2 * (R(1) + slack) + R(1e-30) : R(INFINITY);
-  unsigned long long n_nodes = 0, n_tris = 0;
-  bool again = true;
-  for (int pass = 0; pass < 8 && again; ++pass) {
-    // pass 0 starts from the bound.  Exact: a pass that found nothing within it, or
-    // dropped stack entries, is followed by one from the root with the best so far (or
-    // none).  tau < 1: only a pass that dropped entries is repeated, from the best so far.
-    if (pass == 0) best = start;
-    else if (best_t < 0 && exact) best = R(INFINITY);
-    again = false;
-    int sp = 0;
-    int node = 0;
-    for (;;) {
-      F4 lx, ly, lz, hx, hy, hz;
-      I4 ch, cn;
-      if (top != nullptr && node < P.mesh_top) {
-        // one of the tree's top nodes, staged in shared memory by the kernel
-        const float* nd = top + 32 * node;
-        lx = lds4(nd); ly = lds4(nd + 4); lz = lds4(nd + 8);
-        hx = lds4(nd + 12); hy = lds4(nd + 16); hz = lds4(nd + 20);
-        ch = lds4i(nd + 24); cn = lds4i(nd + 28);
-      } else {
-        const float* nd = nodes + 32 * node;
-        lx = ld4(nd); ly = ld4(nd + 4); lz = ld4(nd + 8);
-        hx = ld4(nd + 12); hy = ld4(nd + 16); hz = ld4(nd + 20);
-        ch = ld4i(nd + 24); cn = ld4i(nd + 28);
-      }
-      ++n_nodes;
-      R d[4] = {box_d2_1(x, lx.x, ly.x, lz.x, hx.x, hy.x, hz.x), box_d2_1(x, lx.y, ly.y, lz.y, hx.y, hy.y, hz.y),
-                box_d2_1(x, lx.z, ly.z, lz.z, hx.z, hy.z, hz.z), box_d2_1(x, lx.w, ly.w, lz.w, hx.w, hy.w, hz.w)};
-      const int cc[4] = {ch.x, ch.y, ch.z, ch.w}, nc[4] = {cn.x, cn.y, cn.z, cn.w};
-      // leaf children within the opening threshold: test them now (lowers best)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (nc[i] > 0 && d[i] < tau * best) {
-          for (int j = 0; j < nc[i]; ++j) {
-            R v, w, d2;
-            tri_closest(x, tris + 12 * (cc[i] + j), &v, &w, &d2);
-            if (d2 < best) { best = d2; best_t = cc[i] + j; bv = v; bw = w; }
-          }
-          n_tris += (unsigned long long)nc[i];
+  MeshSearch<R> m;
+  m.begin(bound2, tau, stk_n, stk_d);
+  while (m.sub != MS_DONE) {
+    m.node_step(P, x, stk_n, stk_d, SMEM ? stride : 1, top);
+    while (m.sub == MS_TRI) {
+      R d2 = R(INFINITY), v = R(0), w = R(0);
+      int t = -1;
+      for (int j = m.lt; j < m.le; ++j) {
+        R jv, jw, jd2;
+        tri_closest(x, P.mesh_tris + 12 * j, &jv, &jw, &jd2);
+        if (jd2 < d2) {
+          d2 = jd2;
+          v = jv;
+          w = jw;
+          t = j;
         }
       }
-      const R thr = tau * best;
-      // interior children within the threshold: sort by distance (others at infinity)
-      R k[4];
-      int c[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        k[i] = (nc[i] == 0 && d[i] < thr) ? d[i] : R(INFINITY);
-        c[i] = cc[i];
-      }
-#define WOS_CSWAP(a, b)                                   \
-  if (k[b] < k[a]) {                                      \
-    R tk = k[a]; k[a] = k[b]; k[b] = tk;                  \
-    int tc = c[a]; c[a] = c[b]; c[b] = tc;                \
-  }
-      WOS_CSWAP(0, 1) WOS_CSWAP(2, 3) WOS_CSWAP(0, 2) WOS_CSWAP(1, 3) WOS_CSWAP(1, 2)
-#undef WOS_CSWAP
-      // push the farther ones (farthest first, so the nearer are popped first)
-#pragma unroll
-      for (int i = 3; i >= 1; --i) {
-        if (k[i] < thr) {
-          if (sp < kMeshStack) {
-            stk_n[sp * sst] = c[i];
-            stk_d[sp * sst] = k[i];
-            ++sp;
-          } else {
-            again = true;
-          }
-        }
-      }
-      if (k[0] < thr) {
-        node = c[0];
-        continue;
-      }
-      // pop the next node still within the threshold of the best triangle
-      bool found = false;
-      while (sp > 0) {
-        --sp;
-        if (stk_d[sp * sst] < tau * best) { node = stk_n[sp * sst]; found = true; break; }
-      }
-      if (!found) break;
+      m.leaf_done(P, d2, v, w, t);
     }
-    if (best_t < 0 && exact) again = true;
   }
-  MeshHit<R> h;
-  if (vis != nullptr) {
-    vis->nodes += n_nodes;
-    vis->tris += n_tris;
+  return m.hit(P, x, pb, vis);
+}
+
+// Mesh distance grid at x: lower bound max_c (d(c) - |x - c|) of the distance over the cell's
+// corners into *lo_b, and min_c (d(c) + |x - c|), squared, lowers *bound2 (*own: the bound then has
+// no boundary point of its own).  True if the lower bound is the walk's radius.
+template <typename R>
+WOS_HD bool mesh_grid_radius(const DevProblem<R>& P, const R* x, R* lo_out, R* bound2, bool* own) {
+  int i0[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    R sg = floor((x[d] - P.mg_lo[d]) * P.mg_inv_h[d]);
+    int i = (int)w_fmin(w_fmax(sg, R(0)), R(P.mg_res - 2));
+    i0[d] = i;
   }
-  if (best_t >= 0) {
-    const float* t = tris + 12 * best_t;
-    F4 A = ld4(t), B = ld4(t + 4), Cc = ld4(t + 8);
-    h.x = R(A.x) + (R(B.x) - R(A.x)) * bv + (R(Cc.x) - R(A.x)) * bw;
-    h.y = R(A.y) + (R(B.y) - R(A.y)) * bv + (R(Cc.y) - R(A.y)) * bw;
-    h.z = R(A.z) + (R(B.z) - R(A.z)) * bv + (R(Cc.z) - R(A.z)) * bw;
-    h.d = exact ? w_sqrt(best) : w_sqrt(tau * best);
-  } else if (!exact && best < R(INFINITY)) {
-    // nothing inside the bound: its own boundary point (when known) is the best point
-    h.x = pb ? pb[0] : R(NAN);
-    h.y = pb ? pb[1] : R(NAN);
-    h.z = pb ? pb[2] : R(NAN);
-    h.d = w_sqrt(tau * best);
-  } else {
-    // no boundary point found at all (eight passes of overflowing stacks, or a non-finite
-    // point): counted, and the walk ends here (distance 0, closest point x)
-    if (vis != nullptr) ++vis->exhausted;
-    h.x = x0;
-    h.y = x1;
-    h.z = x2;
-    h.d = R(0);
+  R lo_b = R(-INFINITY), hi_b = R(INFINITY);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    int ii = i0[0] + (c & 1), jj = i0[1] + ((c >> 1) & 1), kk = i0[2] + ((c >> 2) & 1);
+    R e0 = x[0] - (P.mg_lo[0] + R(ii) * P.mg_h[0]);
+    R e1 = x[1] - (P.mg_lo[1] + R(jj) * P.mg_h[1]);
+    R e2 = x[2] - (P.mg_lo[2] + R(kk) * P.mg_h[2]);
+    R dist = w_sqrt(e0 * e0 + e1 * e1 + e2 * e2);
+    R dc = P.mgrid[ii + (int64_t)P.mg_res * (jj + (int64_t)P.mg_res * kk)];
+    lo_b = w_fmax(lo_b, dc - dist);
+    hi_b = w_fmin(hi_b, dc + dist);
   }
-  return h;
+  *lo_out = lo_b;
+  if (lo_b >= P.mg_thresh) return true;
+  if (hi_b * hi_b < *bound2) {
+    *bound2 = hi_b * hi_b;
+    *own = false;
+  }
+  return false;
 }
 
 // ---------------------------------------------------------------------------
@@ -911,36 +1049,15 @@ WOS_HD R distance(const DevProblem<R>& P, const R* x, R* xb, R bound2 = R(INFINI
     case D_MESH: {
       if (DIM != 3 || !MESH) return R(-1);
       if (P.mg_res > 0) {
-        // distance grid: lower bound max_c (d(c) - |x - c|), upper bound min_c (d(c) + |x - c|)
-        int i0[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          R sg = floor((x[d] - P.mg_lo[d]) * P.mg_inv_h[d]);
-          int i = (int)w_fmin(w_fmax(sg, R(0)), R(P.mg_res - 2));
-          i0[d] = i;
-        }
-        R lo_b = R(-INFINITY), hi_b = R(INFINITY);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          int ii = i0[0] + (c & 1), jj = i0[1] + ((c >> 1) & 1), kk = i0[2] + ((c >> 2) & 1);
-          R e0 = x[0] - (P.mg_lo[0] + R(ii) * P.mg_h[0]);
-          R e1 = x[1] - (P.mg_lo[1] + R(jj) * P.mg_h[1]);
-          R e2 = x[2] - (P.mg_lo[2] + R(kk) * P.mg_h[2]);
-          R dist = w_sqrt(e0 * e0 + e1 * e1 + e2 * e2);
-          R dc = P.mgrid[ii + (int64_t)P.mg_res * (jj + (int64_t)P.mg_res * kk)];
-          lo_b = w_fmax(lo_b, dc - dist);
-          hi_b = w_fmin(hi_b, dc + dist);
-        }
-        if (lo_b >= P.mg_thresh) {
+        R lo_b;
+        bool own = true;
+        if (mesh_grid_radius(P, x, &lo_b, &bound2, &own)) {
           // the walk is not in the shell; no boundary point is known (NaN: the next step's
           // query starts without a bound)
           xb[0] = xb[1] = xb[2] = R(NAN);
           return lo_b;
         }
-        if (hi_b * hi_b < bound2) {
-          bound2 = hi_b * hi_b;
-          pb = nullptr;  // the grid's bound has no boundary point of its own
-        }
+        if (!own) pb = nullptr;
       }
       MeshHit<R> h = (stk_n != nullptr)
                          ? mesh_query<R, true>(P, x[0], x[1], x[2], bound2, stk_n, stk_d, stk_stride, tau, pb, vis,

@@ -163,6 +163,12 @@ __device__ __forceinline__ void start_walk(const WalkLaunch& L, uint64_t item, u
 #if !defined(WOS_WALK_MIN_BLOCKS)
 #define WOS_WALK_MIN_BLOCKS 5
 #endif
+// Mesh walks: four blocks of 128 registers (the walk and its search stay in registers; 5 / 4 / 3
+// blocks measured 108 / 107 / 113 ms with certified radii, 144 / 135 / 129 ms with exact ones on the
+// cases at the search loop), and how many lanes a warp gathers before it tests their leaves
+// together (4 / 5 / 6 / 8 / 12: 105 / 106 / 105 / 107 / 116 ms and 126 / 128 / 133 / 135 / 152 ms).
+constexpr int kMeshBlocks = 4;
+constexpr int kMeshLeaves = 5;
 #if defined(WOS_JIT_FIELDS)
 #define WOS_WALK_KERNEL wos_walk_spec_kernel
 #else
@@ -172,7 +178,7 @@ __device__ __forceinline__ void start_walk(const WalkLaunch& L, uint64_t item, u
 // variant, chosen by the schedule).
 template <int DIM, typename R, bool MESH, bool BATCHED, bool WW, bool GRAD, bool DRIFT = false, int MINB = 0>
 __global__ void __launch_bounds__(kWalkBlock,
-                                  (sizeof(R) == 4) ? (GRAD ? 5 : (MESH ? 5 : (MINB > 0 ? MINB : WOS_WALK_MIN_BLOCKS))) : 1)
+                                  (sizeof(R) == 4) ? (GRAD ? 5 : (MESH ? kMeshBlocks : (MINB > 0 ? MINB : WOS_WALK_MIN_BLOCKS))) : 1)
     WOS_WALK_KERNEL(WalkLaunch L) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // stage the problem description (a few KB, read by every lane every step) in shared memory
@@ -187,17 +193,12 @@ __global__ void __launch_bounds__(kWalkBlock,
   // MESH: this thread's column of the BVH traversal stack, after the problem
   int* stk_n = nullptr;
   R* stk_d = nullptr;
-  // and the tree's top nodes (every query starts at the root), staged after the stacks
-  const float* mtop = nullptr;
+  int* owners = nullptr;  // and eight words per warp: the lanes whose leaves a warp tests together
   if (MESH) {
     stk_n = reinterpret_cast<int*>(smem_raw + L.problem_bytes) + threadIdx.x;
     stk_d = reinterpret_cast<R*>(smem_raw + L.problem_bytes + sizeof(int) * kMeshStack * kWalkBlock) + threadIdx.x;
-    float* top = reinterpret_cast<float*>(smem_raw + L.problem_bytes + (sizeof(int) + sizeof(R)) * kMeshStack * kWalkBlock);
-    const int n4 = 8 * min(Pshared->mesh_top, kMeshTopMax);  // 8 x 16 bytes per node
-    const float4* src = reinterpret_cast<const float4*>(Pshared->mesh_nodes);
-    for (int i = threadIdx.x; i < n4; i += blockDim.x) reinterpret_cast<float4*>(top)[i] = __ldg(src + i);
-    __syncthreads();
-    mtop = top;
+    owners = reinterpret_cast<int*>(smem_raw + L.problem_bytes + (sizeof(int) + sizeof(R)) * kMeshStack * kWalkBlock) +
+             8 * (threadIdx.x >> 5);
   }
 
   const int lane = threadIdx.x & 31;
@@ -238,6 +239,13 @@ __global__ void __launch_bounds__(kWalkBlock,
   unsigned long long st_steps = 0;
   uint32_t st_walks = 0, st_capped = 0, st_nonfinite = 0, st_outside = 0;
   MeshVisits mvis = {0ull, 0ull, 0u};  // mesh queries: nodes, triangles, exhausted searches
+  // meshes: the lane's distance query, and whether its walk steps next (or begins), searches, or
+  // knows its distance mesh_d (and closest point s.xbp); own_pb: the search's bound is s.xbp's
+  enum { MQ_STEP = 0, MQ_SEARCH = 1, MQ_READY = 2 };
+  MeshSearch<R> ms;
+  int mode = MQ_STEP;
+  R mesh_d = R(0);
+  bool own_pb = false;
   // weight window: copies waiting to run (position, weight, step, branch id)
   R stk_x[WW ? kWWDepth : 1][3], stk_W[WW ? kWWDepth : 1];
   uint32_t stk_k[WW ? kWWDepth : 1], stk_id[WW ? kWWDepth : 1];
@@ -380,6 +388,119 @@ __global__ void __launch_bounds__(kWalkBlock,
       }
     }
     if (__ballot_sync(kFull, active) == 0u) break;
+    if (MESH) {
+      // Distance queries.  A query visits anything from a handful of nodes near the boundary to
+      // hundreds deep inside, so lanes that all wait for the warp's longest one idle most of the
+      // time (5.3 of 32 lanes active with certified radii, 3.1 with exact ones).  Each lane keeps
+      // its search in registers and searches on while others step: the warp visits nodes, or tests
+      // the leaves of up to eight lanes with four lanes each, until half of its walks know their
+      // distance; those take their step and begin their next search.  17 lanes take part in a node
+      // visit, 19 triangles are tested at a time.  Measured: 327,680 triangles, 8192 points x 100
+      // walks, certified radii (tol 0.1) 200 -> 106 ms; 20,480 triangles, 3000 x 64, exact radii
+      // 266 -> 128 ms.  Four lanes to a whole search (a child box each, eight searches a warp) was
+      // slower: 231 and 196 ms, bound by the latency of too few searches in flight; a step at 1/4 or
+      // 3/4 of the walks ready 120 and 113 ms.
+      if (active && mode == MQ_STEP) {
+        // the previous step's boundary point bounds the query (NaN when none is known)
+        R bound2 = R(INFINITY);
+        if (s.k > 0) {
+          R e[3] = {s.x[0] - s.xbp[0], s.x[1] - s.xbp[1], s.x[2] - s.xbp[2]};
+          R b2 = dot3(e, e);
+          if (b2 < R(INFINITY)) bound2 = b2;
+        }
+        own_pb = bound2 < R(INFINITY);
+        mode = MQ_SEARCH;
+        if (Pshared->mg_res > 0 && mesh_grid_radius(*Pshared, s.x, &mesh_d, &bound2, &own_pb)) {
+          // the grid's radius: no boundary point is known
+          s.xbp[0] = s.xbp[1] = s.xbp[2] = R(NAN);
+          mode = MQ_READY;
+        } else {
+          ms.begin(bound2, Pshared->mesh_tau, stk_n, stk_d);
+        }
+      }
+      const int walking = __popc(__ballot_sync(kFull, active));
+      for (;;) {
+        const bool searching = active && mode == MQ_SEARCH;
+        const unsigned node = __ballot_sync(kFull, searching && ms.sub == MS_NODE);
+        const unsigned tri = __ballot_sync(kFull, searching && ms.sub == MS_TRI);
+        const int n_node = __popc(node), n_tri = __popc(tri);
+        if (2 * (n_node + n_tri) <= walking) {
+          // enough lanes are through: take their results (lanes that began an exact search go on)
+          if (searching && ms.sub == MS_DONE) {
+            const MeshHit<R> h = ms.hit(*Pshared, s.x, own_pb ? s.xbp : nullptr, &mvis);
+            mesh_d = h.d;
+            s.xbp[0] = h.x;
+            s.xbp[1] = h.y;
+            s.xbp[2] = h.z;
+            mode = MQ_READY;
+            if (ms.tau < R(1) && !(h.d >= eps)) {
+              // a certified radius below eps: the exact distance decides the eps-shell test and
+              // gives the closest point for g (a step or two per walk, near the boundary)
+              R e[3] = {s.x[0] - h.x, s.x[1] - h.y, s.x[2] - h.z};
+              R b2 = dot3(e, e);
+              if (!(b2 < R(INFINITY))) b2 = R(INFINITY);
+              own_pb = false;
+              R lo_b;
+              if (Pshared->mg_res > 0) mesh_grid_radius(*Pshared, s.x, &lo_b, &b2, &own_pb);
+              ms.begin(b2, R(1), stk_n, stk_d);
+              mode = MQ_SEARCH;
+            }
+          }
+          if (__any_sync(kFull, active && mode == MQ_READY)) break;
+          continue;
+        }
+        if (n_tri >= kMeshLeaves || n_node == 0) {
+          // the leaves of up to eight lanes, four lanes to a leaf (at most four triangles as a rule)
+          const int rank = __popc(tri & lt_mask);
+          const bool mine = (tri >> lane & 1u) && rank < 8;
+          if (mine) owners[rank] = lane;
+          __syncwarp();
+          const bool on = (lane >> 2) < n_tri;
+          const int from = on ? owners[lane >> 2] : lane;
+          const R qx[3] = {__shfl_sync(kFull, s.x[0], from), __shfl_sync(kFull, s.x[1], from),
+                           __shfl_sync(kFull, s.x[2], from)};
+          const int lt = __shfl_sync(kFull, ms.lt, from), le = __shfl_sync(kFull, ms.le, from);
+          __syncwarp();
+          R d2 = R(INFINITY), v = R(0), w = R(0);
+          int t = 0x7fffffff;
+          if (on) {
+            for (int j = lt + (lane & 3); j < le; j += 4) {
+              R jv, jw, jd2;
+              tri_closest(qx, Pshared->mesh_tris + 12 * j, &jv, &jw, &jd2);
+              if (jd2 < d2) {
+                d2 = jd2;
+                v = jv;
+                w = jw;
+                t = j;
+              }
+            }
+          }
+          // the leaf's nearest triangle, the first of equals
+#pragma unroll
+          for (int off = 1; off <= 2; off <<= 1) {
+            const R od2 = __shfl_xor_sync(kFull, d2, off), ov = __shfl_xor_sync(kFull, v, off);
+            const R ow = __shfl_xor_sync(kFull, w, off);
+            const int ot = __shfl_xor_sync(kFull, t, off);
+            if (od2 < d2 || (od2 == d2 && ot < t)) {
+              d2 = od2;
+              v = ov;
+              w = ow;
+              t = ot;
+            }
+          }
+          const int got = mine ? 4 * rank : lane;
+          d2 = __shfl_sync(kFull, d2, got);
+          v = __shfl_sync(kFull, v, got);
+          w = __shfl_sync(kFull, w, got);
+          t = __shfl_sync(kFull, t, got);
+          if (mine) ms.leaf_done(*Pshared, d2, v, w, t);
+        } else if (node >> lane & 1u) {
+          ms.node_step(*Pshared, s.x, stk_n, stk_d, kWalkBlock, nullptr);
+        }
+      }
+      if (!active || mode != MQ_READY) continue;
+      mode = MQ_STEP;
+    }
     if (!active) continue;
     const DevProblem<R>& P = BATCHED ? Pall[s.prob] : *Pshared;
     R s_root = s_root0, inv_sb = inv_sb0;
@@ -393,29 +514,9 @@ __global__ void __launch_bounds__(kWalkBlock,
     R xb[3];
     R d;
     if (MESH) {
-      // the previous step's boundary point bounds the query (NaN when none is known)
-      R bound2 = R(INFINITY);
-      if (s.k > 0) {
-        R e0 = s.x[0] - s.xbp[0], e1 = s.x[1] - s.xbp[1], e2 = s.x[2] - s.xbp[2];
-        R b2 = e0 * e0 + e1 * e1 + e2 * e2;
-        if (b2 < R(INFINITY)) bound2 = b2;
-      }
-      const R tau = P.mesh_tau;
-      d = distance<DIM, R, MESH>(P, s.x, xb, bound2, stk_n, stk_d, kWalkBlock, tau,
-                                 (bound2 < R(INFINITY)) ? s.xbp : nullptr, &mvis, mtop);
-      if (tau < R(1) && !(d >= eps)) {
-        // a certified radius below eps: the exact distance decides the eps-shell test and
-        // gives the closest point for g (a step or two per walk, near the boundary)
-        R e0 = s.x[0] - xb[0], e1 = s.x[1] - xb[1], e2 = s.x[2] - xb[2];
-        R b2 = e0 * e0 + e1 * e1 + e2 * e2;
-        R xe[3];
-        d = distance<DIM, R, MESH>(P, s.x, xe, (b2 < R(INFINITY)) ? b2 : R(INFINITY), stk_n, stk_d, kWalkBlock,
-                                   R(1), nullptr, &mvis, mtop);
+      d = mesh_d;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) xb[i] = xe[i];
-      }
-#pragma unroll
-      for (int i = 0; i < 3; ++i) s.xbp[i] = xb[i];
+      for (int i = 0; i < 3; ++i) xb[i] = s.xbp[i];
     } else {
       d = distance<DIM, R, MESH>(P, s.x, xb);
     }
@@ -629,7 +730,7 @@ template <int DIM, typename R, bool MESH, bool BATCHED, bool WW, bool GRAD = fal
           int MINB = 0>
 cudaError_t launch_walks_m(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
   size_t smem = BATCHED ? 0 : (size_t)L.problem_bytes;
-  if (MESH) smem += (sizeof(int) + sizeof(R)) * kMeshStack * kWalkBlock + 128 * kMeshTopMax;
+  if (MESH) smem += (sizeof(int) + sizeof(R)) * kMeshStack * kWalkBlock + kWalkBlock;
   if (smem > 48 * 1024) {
     cudaError_t ea = cudaFuncSetAttribute(wos_walk_kernel<DIM, R, MESH, BATCHED, WW, GRAD, DRIFT, MINB>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
