@@ -142,6 +142,17 @@ WOS_HD void w_sincospi2(double u, double* s, double* c) {
 }
 WOS_HD float w_fma(float a, float b, float c) { return fmaf(a, b, c); }
 WOS_HD double w_fma(double a, double b, double c) { return fma(a, b, c); }
+// 1 - x^2: FORM 1 fused, 2 with the square rounded first
+template <int FORM>
+WOS_HD float w_one_minus_sq(float x) {
+#if defined(__CUDA_ARCH__)
+  return FORM == 2 ? __fadd_rn(1.0f, -__fmul_rn(x, x)) : fmaf(-x, x, 1.0f);
+#else
+  return 1.0f - x * x;
+#endif
+}
+template <int FORM>
+WOS_HD double w_one_minus_sq(double x) { return 1.0 - x * x; }
 WOS_HD float w_cbrt(float x) { return cbrtf(x); }
 WOS_HD double w_cbrt(double x) { return cbrt(x); }
 WOS_HD float w_expm1(float x) { return expm1f(x); }
@@ -440,6 +451,12 @@ struct FactPoly<R, OFF, K, NT, true> {
 //   |G| = R^2 q(a) with 3D q = (1 - a/sinh a)/a^2, 2D q = (1 - 1/I0(a))/a^2,
 //   P^B = sb |G| = a^2 q(a).
 // ---------------------------------------------------------------------------
+// FORM (here and in Radial3) names the roundings of (1 - e^{-2a}) - 2a e^{-a}: 0 leaves the choice
+// to the compiler, 1 and 2 are w_one_minus_sq's with the rest fused.  They differ in the last bit,
+// but a walk's path depends on every bit; the gradient walks name the form that their kernels have
+// always had (generic 1, specialised 2), so that they stay the same walks however the kernel around
+// them is laid out.
+template <int FORM = 0>
 WOS_HD float green_q3(float a) {
   // q = (1 - a/sinh a)/a^2 = S(a) / (a^2 sinh a), S(a) = sinh a - a.  a < 1: S(a) = a^3 P(a^2)
   // and sinh a = a (1 + a^2 P(a^2)), P(t) = sum t^k/(2k+3)! (the radial CDF's series, which
@@ -449,9 +466,12 @@ WOS_HD float green_q3(float a) {
   const float P = FactPoly<float, 3, 0, 5>::eval(t);
   const float e = w_exp(-a);
   const float qs = w_div(P, 1.0f + t * P);
-  const float ql = w_div((1.0f - e * e) - 2.0f * a * e, t * (1.0f - e * e));
+  const float om = w_one_minus_sq<FORM>(e);
+  const float ql = FORM ? w_div(w_fma(-(2.0f * a), e, om), t * om)
+                      : w_div((1.0f - e * e) - 2.0f * a * e, t * (1.0f - e * e));
   return (a < 1.0f) ? qs : ql;
 }
+template <int FORM = 0>
 WOS_HD double green_q3(double a) {
   if (a < 1.0) {  // (sinh a - a)/(a^2 sinh a) by the series of sinh a - a
     double t = a * a, term = a, s = 0.0;
@@ -495,9 +515,9 @@ WOS_HD double green_q2(double a) {
   return (1.0 - exp(-a) / d_i0s(a)) / (a * a);
 }
 
-template <int DIM, typename R>
+template <int DIM, typename R, int FORM = 0>
 WOS_HD R green_q(R a) {
-  return DIM == 2 ? green_q2(a) : green_q3(a);
+  return DIM == 2 ? green_q2(a) : green_q3<FORM>(a);
 }
 
 // ---------------------------------------------------------------------------
@@ -992,13 +1012,14 @@ struct Radial3 {
   R K;     // units of the series form of the numerator
   R invD;  // 1 / denominator
 
+  template <int FORM = 0>
   WOS_HD void init(R a_) {
     a = a_;
     ea = w_exp(-a);
     const R a2 = a * a;
     const bool sm = a < R(1);
     const R dsm = FactPoly<R, 3, 0, NC>::eval(a2);
-    const R dlg = (R(1) - ea * ea) - R(2) * a * ea;
+    const R dlg = FORM ? w_fma(-(R(2) * a), ea, w_one_minus_sq<FORM>(ea)) : (R(1) - ea * ea) - R(2) * a * ea;
     K = sm ? R(1) : R(2) * ea * a2 * a;
     invD = w_div(R(1), sm ? dsm : dlg);
   }
@@ -1354,7 +1375,7 @@ WOS_HD float table_guess(const float* tab, float a, float u) {
   return v0 + ta * (v1 - v0);
 }
 
-template <int DIM, typename R>
+template <int DIM, typename R, int FORM = 0>
 WOS_HD R sample_radius(R a, R u, int* iters_used = nullptr, const float* tab = nullptr) {
   // FP32: the loop serves only the rare samples outside the table's one-step range (the
   // last t interval, a >= 32); in the flat tail near rho = 1 it may need bisection steps
@@ -1377,7 +1398,7 @@ WOS_HD R sample_radius(R a, R u, int* iters_used = nullptr, const float* tab = n
     R F, p;
     if (DIM == 3) {
       Radial3<R> rad;
-      rad.init(a);
+      rad.template init<FORM>(a);
       rad.eval(g, &F, &p);
     } else {
       radial2_once(a, g, &F, &p);
@@ -1390,7 +1411,7 @@ WOS_HD R sample_radius(R a, R u, int* iters_used = nullptr, const float* tab = n
   }
   if (DIM == 3) {
     Radial3<R> rad;
-    rad.init(a);
+    rad.template init<FORM>(a);
     return newton_inverse(rad, u, g, iters, tol, ftol, iters_used);
   } else {
     Radial2<R> rad;

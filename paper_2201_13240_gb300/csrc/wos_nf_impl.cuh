@@ -156,6 +156,7 @@ __global__ void __launch_bounds__(kNfBlock, (sizeof(R) == 4) ? 4 : 1) wos_nf_ker
     U4 r1 = U4{0u, 0u, 0u, 0u};
     R pRR = R(1);
     bool ended = false;
+#pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
       if (phase == 0) {
         // ---- a new ball: distance query, exit point, first boundary term ----

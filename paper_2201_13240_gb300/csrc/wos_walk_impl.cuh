@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kWalkBlock,
   // small solves: one walk per lane and claim, so that the walks of a launch that does not
   // fill the chip run side by side; their sums are left to walk_sum_kernel
   const bool spread = sizeof(R) == 4 && !GRAD && L.item_acc != nullptr && total <= kSpreadItems;
-  if (spread) chunk = 32;
+  if (spread || (GRAD && total <= kSpreadItems)) chunk = 32;
   uint64_t chunk_next = 0, chunk_end = 0;
   uint32_t cur_p = 0, cur_prob = 0;
   const uint64_t magic = (L.walks_uniform > 0) ? ~0ull / (uint64_t)L.walks_uniform : 0ull;
@@ -343,7 +343,12 @@ __global__ void __launch_bounds__(kWalkBlock,
   // divergent blocks (end and regeneration, run by one or two lanes) then run about once per
   // kDeferLanes walk ends instead of in most iterations, while the waiting lanes sit out a
   // few steps.
-  constexpr bool DEFER = !WW && !GRAD && !MESH;
+  constexpr bool DEFER = !WW && !MESH;
+#if defined(WOS_JIT_FIELDS)
+  constexpr int kForm = GRAD ? 2 : 0;  // see green_q3
+#else
+  constexpr int kForm = GRAD ? 1 : 0;
+#endif
   bool pend = false, pcap = false;
   R pgam = R(0), pxb[3] = {R(0), R(0), R(0)};
 
@@ -560,7 +565,7 @@ __global__ void __launch_bounds__(kWalkBlock,
       }
     }
     R a = s_root * dd;
-    R q = green_q<DIM, R>(a);
+    R q = green_q<DIM, R, kForm>(a);
     R Gn = dd * dd * q;        // |G| on the ball of radius d
     R PB = a * a * q;          // sigma_bar |G|, probability of the volume term
     // DRIFT (every ball, G/|G| weight 0.97: the weight ratios multiply along the walk) and
@@ -572,7 +577,7 @@ __global__ void __launch_bounds__(kWalkBlock,
     const float* tab = (sizeof(R) == 4) ? L.radial_tab : nullptr;
     const bool mix = DRIFT || (GRAD && s.k == 0);
     const R lam = DRIFT ? R(0.97) : R(0.5);
-    R rho = sample_radius<DIM, R>(a, mix ? ((ur < lam) ? ur / lam : R(0.5)) : ur, nullptr, tab);
+    R rho = sample_radius<DIM, R, kForm>(a, mix ? ((ur < lam) ? ur / lam : R(0.5)) : ur, nullptr, tab);
     if (mix) rho = mix_radius_weight<DIM, R>(a, ur, rho, lam, &mixw);
     R r = rho * dd;
     // coefficient point: y for a step; the walk's own point when it ends (gamma(x_n))
