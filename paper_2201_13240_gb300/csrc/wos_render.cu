@@ -40,6 +40,94 @@ __device__ double sd_domain(const DevProblem<double>& P, const double* x) {
   return -distance<3, double, false>(P, x, xb);  // signed distance, negative inside
 }
 
+// A CSG list in FP32, with a bound of the FP32 distances' error: the sphere tracer asks it which
+// primitive decides the signed distance, and evaluates that one alone in FP64.
+//
+// What bounds the view is the FP64 pipe (1/64 of the FP32 lanes' rate here): every step of a ray
+// evaluated the plane and every primitive in FP64, some 25 operations each with a square root.  The
+// FP32 pass costs a fraction of that; where its intervals do not tell the winner (a crease, a far-off
+// point) the whole list is evaluated in FP64 as before, so every step's length, and the image, is
+// the same.  Measured (1280 x 720, five primitives): 5.70 -> 2.48 ms, FP64 pipe 56 % busy; more
+// resident blocks by spilling (3, 4 or 5 of 256 threads) 2.8, 2.9 and 4.3 ms.
+struct CsgF32 {
+  CsgNode<float> node[kMaxCsg];
+  float size[kMaxCsg];   // largest parameter, times (1 + its normal's) for a half-space
+};
+
+__device__ void csg_load_f32(const DevProblem<double>& P, CsgF32* C) {
+  const int n = P.domain_kind == D_CSG ? P.ncsg : 0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    C->node[i].prim = P.csg[i].prim;
+    C->node[i].op = P.csg[i].op;
+    float m = 0.0f;
+    for (int k = 0; k < 8; ++k) {
+      C->node[i].p[k] = (float)P.csg[i].p[k];
+      m = fmaxf(m, fabsf(C->node[i].p[k]));
+    }
+    C->size[i] = m * (P.csg[i].prim == C_HALFSPACE ? 1.0f + m : 1.0f);
+  }
+}
+
+// The interval [lo, hi] of csg_sdf at a point and the primitive that gives it, -1 where that is open
+// (an unbounded interval if some distance is not finite).  xf is the point in FP32, off by a few
+// roundings of numbers no larger than X (>= the sum of its coordinates' magnitudes).  A primitive's
+// FP32 distance takes at most a few dozen roundings of numbers no larger than X plus its parameters
+// (a half-space: times its normal's length): 64 units of 2^-24 bound its error.
+__device__ int csg_decide(const CsgF32& C, int n, const float* xf, float X, float* lo, float* hi) {
+  float l = 0.0f, h = 0.0f;
+  int who = 0;
+  bool finite = true;
+  for (int i = 0; i < n; ++i) {
+    float g[3];
+    const int op = C.node[i].op;
+    float s = csg_prim<3, float>(C.node[i], xf, g);
+    const float grow = C.node[i].prim == C_HALFSPACE ? 1.0f + C.size[i] : 1.0f;
+    const float e = 64.0f * 5.9604645e-8f * (X * grow + C.size[i]);
+    if (i > 0 && op == C_SUBTRACT) s = -s;
+    const float a = s - e, b = s + e;
+    finite = finite && fabsf(a) < INFINITY && fabsf(b) < INFINITY;
+    if (i == 0) {
+      l = a;
+      h = b;
+    } else if (op == C_UNION) {   // the smaller
+      if (b < l) {
+        who = i;
+        l = a;
+        h = b;
+      } else if (!(a > h)) {
+        who = -1;
+        l = fminf(l, a);
+        h = fminf(h, b);
+      }
+    } else {                      // the larger
+      if (a > h) {
+        who = i;
+        l = a;
+        h = b;
+      } else if (!(b < l)) {
+        who = -1;
+        l = fmaxf(l, a);
+        h = fmaxf(h, b);
+      }
+    }
+  }
+  *lo = finite ? l : -INFINITY;
+  *hi = finite ? h : INFINITY;
+  return finite ? who : -1;
+}
+
+// sd_domain through csg_decide
+__device__ double sd_decided(const DevProblem<double>& P, const CsgF32& C, const double* x) {
+  if (P.domain_kind != D_CSG) return sd_domain(P, x);
+  const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
+  float lo, hi;
+  const int who = csg_decide(C, P.ncsg, xf, fabsf(xf[0]) + fabsf(xf[1]) + fabsf(xf[2]), &lo, &hi);
+  if (who < 0) return sd_domain(P, x);
+  double g[3];
+  const double s = csg_prim<3, double>(P.csg[who], x, g);
+  return (who > 0 && P.csg[who].op == C_SUBTRACT) ? -s : s;
+}
+
 __device__ void colour_map(double t, double* c) {
   // a blue - white - red map on [0, 1]
   t = fmin(fmax(t, 0.0), 1.0);
@@ -60,6 +148,10 @@ __device__ void put(uint8_t* rgba, int64_t i, const double* c) {
 __global__ void render3_kernel(const DevProblem<double>* Pg, View3 V, const double* sum, const int64_t* count,
                                uint8_t* rgba, float* value, float* depth) {
   const DevProblem<double>& P = *Pg;
+  __shared__ CsgF32 C;
+  csg_load_f32(P, &C);
+  __syncthreads();
+  const bool csg = P.domain_kind == D_CSG;
   int64_t npx = (int64_t)V.width * V.height;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < npx; i += (int64_t)gridDim.x * blockDim.x) {
     int px = (int)(i % V.width), py = (int)(i / V.width);
@@ -76,13 +168,48 @@ __global__ void render3_kernel(const DevProblem<double>* Pg, View3 V, const doub
     float val = NAN, dep = INFINITY;
     // sphere-trace max(sdf_domain, sdf_keep): the domain behind the plane
     double t = 0.0, tmax = 1e3 * V.scale;
+    float eyef[3], dirf[3], nf[3], orgf[3], eye1 = 0.0f, org1 = 0.0f;
+    for (int k = 0; k < 3; ++k) {
+      eyef[k] = (float)V.eye[k];
+      dirf[k] = (float)dir[k];
+      nf[k] = (float)V.n[k];
+      orgf[k] = (float)V.org[k];
+      eye1 += fabsf(eyef[k]);
+      org1 += fabsf(orgf[k]);
+    }
     const double tol = 1e-5 * V.scale;
     for (int it = 0; it < 512 && t < tmax; ++it) {
       double x[3];
       for (int k = 0; k < 3; ++k) x[k] = V.eye[k] + t * dir[k];
-      double sd = sd_domain(P, x);
-      double sp = 0.0;  // > 0 on the eye's side of the plane: cut away
-      for (int k = 0; k < 3; ++k) sp += V.n[k] * (x[k] - V.org[k]);
+      // which of the domain's and the plane's distance is the larger, in FP32 where that suffices
+      bool plane = true, domain = true;  // may be
+      int who = -1;
+      if (csg) {
+        const float tf = (float)t, X = eye1 + 1.75f * fabsf(tf);
+        float xf[3], spf = 0.0f, lo, hi;
+        for (int k = 0; k < 3; ++k) {
+          xf[k] = eyef[k] + tf * dirf[k];
+          spf += nf[k] * (xf[k] - orgf[k]);
+        }
+        who = csg_decide(C, P.ncsg, xf, X, &lo, &hi);
+        const float e = 64.0f * 5.9604645e-8f * (X + org1);
+        plane = !(spf + e < lo);
+        domain = !(hi < spf - e);
+      }
+      double sd = -INFINITY, sp = -INFINITY;
+      if (plane) {  // > 0 on the eye's side of the plane: cut away
+        sp = 0.0;
+        for (int k = 0; k < 3; ++k) sp += V.n[k] * (x[k] - V.org[k]);
+      }
+      if (domain) {
+        if (who >= 0) {
+          double g[3];
+          sd = csg_prim<3, double>(P.csg[who], x, g);
+          if (who > 0 && P.csg[who].op == C_SUBTRACT) sd = -sd;
+        } else {
+          sd = sd_domain(P, x);
+        }
+      }
       double s = fmax(sd, sp);
       if (s < tol) {
         dep = (float)t;
@@ -114,7 +241,7 @@ __global__ void render3_kernel(const DevProblem<double>* Pg, View3 V, const doub
             double xp[3] = {x[0], x[1], x[2]}, xm[3] = {x[0], x[1], x[2]};
             xp[k] += h;
             xm[k] -= h;
-            g[k] = sd_domain(P, xp) - sd_domain(P, xm);
+            g[k] = sd_decided(P, C, xp) - sd_decided(P, C, xm);
           }
           double gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]) + 1e-300;
           double lam = 0.0;
