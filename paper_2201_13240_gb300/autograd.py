@@ -60,6 +60,11 @@ class CoefficientSolve(torch.autograd.Function):
         ctx, prob, walks, eps, sigma_bar, seed, precision, sshape, ashape = fctx.args
         gu = grad_mean.contiguous().to(torch.float64)
         gs = ga = None
+        if sshape is not None and ashape is not None and all(fctx.needs_input_grad[:2]):
+            # one replay of the walks serves both
+            gs, ga = ctx.adjoint(prob, pts, walks, eps, sigma_bar, gu, sigma_nodes=sshape.numel(),
+                                 alpha_nodes=ashape.numel(), seed=seed, precision=precision)
+            return gs.view(sshape), ga.view(ashape), None, None, None, None, None, None, None, None
         if sshape is not None and fctx.needs_input_grad[0]:
             g = torch.zeros(sshape, dtype=torch.float64, device=pts.device)
             ctx.adjoint_sigma(prob, pts, walks, gu, g.view(-1), eps, sigma_bar, seed=seed, precision=precision)

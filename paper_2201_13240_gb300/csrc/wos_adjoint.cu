@@ -3,6 +3,14 @@
 
 namespace wos {
 
+size_t adjoint_smem(const AdjLaunch& L, int real_bytes) {
+  size_t smem = (size_t)L.problem_bytes;
+  if (L.pass == 2 && L.mode != ADJ_SIGMA)
+    smem += (kAdjBlock / 32) * (real_bytes == 8 ? sizeof(AdjStage<double>) : sizeof(AdjStage<float>)) +
+            (size_t)L.priv_nodes * (size_t)real_bytes;
+  return smem;
+}
+
 cudaError_t launch_adjoint_f32(const AdjLaunch& L, int num_sms, cudaStream_t stream) {
   return (L.dim == 2) ? launch_adjoint_t<2, float>(L, num_sms, stream) : launch_adjoint_t<3, float>(L, num_sms, stream);
 }
@@ -11,7 +19,7 @@ cudaError_t launch_adjoint_f32(const AdjLaunch& L, int num_sms, cudaStream_t str
 cudaError_t launch_adjoint_kernel(const AdjLaunch& L, cudaKernel_t kernel, int real_bytes, int num_sms,
                                   cudaStream_t stream) {
   const void* fn = reinterpret_cast<const void*>(kernel);
-  size_t smem = (size_t)L.problem_bytes + ((L.alpha && L.pass == 2) ? (size_t)L.priv_nodes * (size_t)real_bytes : 0);
+  const size_t smem = adjoint_smem(L, real_bytes);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -77,69 +77,89 @@ __device__ __forceinline__ void grid_scatter(const DevField<R>& F, const R* y, R
   }
 }
 
-// add vN N_m + vG . grad N_m + vL Lap N_m at y to grad[m] over the 4^DIM nodes of
-// the cubic B-spline support (indices clamped as in grid_bspline)
-// grad is indexed j0 + s1 j1 + s2 j2: the grid's own layout in global memory, a padded one
-// (s1 = res0 + 1, s2 = s1 res1 + 1) for the per-CTA copy in shared memory, which spreads the
-// rows of one support over different banks.
+// The lanes' scatters of one iteration, staged per warp: for lane e and control a of an axis the basis
+// value b, the axis' combination c of value and derivatives (below) and the clamped control's offset
+// at tap[(4 axis + a) * 33 + e].  The row of 33 keeps the reads of one lane's four entries of an axis
+// in different banks.
+template <typename R>
+struct alignas(16) AdjTap {
+  R b, c;
+  int off;
+};
+template <typename R>
+struct AdjStage {
+  AdjTap<R> tap[12 * 33];
+};
+
+// Add vN N_m + vG . grad N_m + vL Lap N_m at y to grad[m] over the 4^DIM nodes of the cubic
+// B-spline support (indices clamped as in grid_bspline), for every lane of the warp that wants
+// it; all lanes call.  grad is indexed j0 + s1 j1 + s2 j2: the grid's own layout in global memory, or
+// the per-CTA copy's (adj_strides).
+//
+// With B, B', B'' the basis and its derivatives along an axis, the tap of controls (i, j, k) is
+//   Bz (X By + Bx Y) + Z Bx By,   X = vN Bx + vG_x Bx' + vL Bx'',  Y, Z likewise without vN,
+// so a point needs two numbers per axis and control.
+//
+// What bounds it: the instructions of 64 taps and their atomics (compare-and-swap loops) per step.
+// Lane by lane (rows visited in an order rotated by the lane) a step took ~2,000 thread instructions
+// at 21 active lanes, and the lanes' unrelated addresses met in the same banks.  Here the warp takes
+// the lanes' points one after another, two taps a lane (2D: two points, a tap a lane), with every
+// lane active and the 32 atomics of an instruction in 32 banks.  Measured (4096 sensors x 512 walks,
+// 16^3 controls, FP32): the alpha gradient 17.3 -> 14.2 ms (generic
+// kernels 21.8 -> 18.9 ms).  Without the atomics 12.3 ms.
 template <int DIM, typename R, typename A>
-__device__ void bspline_scatter(const DevField<R>& F, const R* y, R vN, const R* vG, R vL, A* grad, int64_t s1,
-                                int64_t s2) {
-  int ib[3] = {0, 0, 0};
-  R B[3][4], B1[3][4], B2[3][4];
+__device__ void bspline_scatter(const DevField<R>& F, const R* y, bool want, R vN, const R* vG, R vL, A* grad,
+                                int64_t s1, int64_t s2, AdjStage<R>* st) {
+  unsigned todo = __ballot_sync(0xffffffffu, want);
+  if (todo == 0u) return;
+  const int lane = threadIdx.x & 31;
+  if (want) {
+    // offsets fit 32 bits: grids stay far below 2^31 nodes
+    const int stride[3] = {1, (int)s1, (int)s2};
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
+    for (int d = 0; d < DIM; ++d) {
+      R B[4], B1[4], B2[4];
+      const R s = (y[d] - F.lo[d]) * F.inv_h[d];
+      const R fs = floor(s);
+      bspline_w(s - fs, B, B1, B2);
+      const int ib = (int)fs - 1;
+      const R c1 = vG[d] * F.inv_h[d], c2 = vL * (F.inv_h[d] * F.inv_h[d]);
 #pragma unroll
-    for (int a = 0; a < 4; ++a) { B[d][a] = (a == 0) ? R(1) : R(0); B1[d][a] = R(0); B2[d][a] = R(0); }
-  }
-#pragma unroll
-  for (int d = 0; d < DIM; ++d) {
-    R s = (y[d] - F.lo[d]) * F.inv_h[d];
-    R fs = floor(s);
-    ib[d] = (int)fs - 1;
-    bspline_w(s - fs, B[d], B1[d], B2[d]);
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      B1[d][a] *= F.inv_h[d];
-      B2[d][a] *= F.inv_h[d] * F.inv_h[d];
+      for (int a = 0; a < 4; ++a)
+        st->tap[(4 * d + a) * 33 + lane] = AdjTap<R>{B[a], (d == 0 ? vN * B[a] : R(0)) + c1 * B1[a] + c2 * B2[a],
+                                                     stride[d] * min(max(ib + a, 0), F.res[d] - 1)};
     }
   }
-  // clamped control indices per axis, once: x offsets and the row / plane offsets (32-bit:
-  // grids stay far below 2^31 nodes)
-  const int t1 = (int)s1, t2 = (int)s2;
-  int o0[4], o1[4], o2[4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    o0[a] = min(max(ib[0] + a, 0), F.res[0] - 1);
-    o1[a] = t1 * min(max(ib[1] + a, 0), F.res[1] - 1);
-    o2[a] = (DIM == 3) ? t2 * min(max(ib[2] + a, 0), F.res[2] - 1) : 0;
-  }
-  // Rows (c1, c2) of the support are visited in an order rotated by the lane, so lanes
-  // whose points share a cell (walks of one point start together) add to different
-  // addresses at the same time instead of serialising on one.
-  auto sel4 = [](const R* v, int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : (i == 2 ? v[2] : v[3])); };
-  auto sel4i = [](const int* v, int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : (i == 2 ? v[2] : v[3])); };
-  const int nrows = (DIM == 3) ? 16 : 4;
-  const int rot = (int)(threadIdx.x & 31);
-  for (int k = 0; k < nrows; ++k) {
-    const int r = (k + rot) & (nrows - 1);
-    const int c1 = r & 3, c2 = (DIM == 3) ? (r >> 2) : 0;
-    const R b1 = sel4(B[1], c1), d1 = sel4(B1[1], c1), e1 = sel4(B2[1], c1);
-    const R b2 = (DIM == 3) ? sel4(B[2], c2) : R(1), d2 = (DIM == 3) ? sel4(B1[2], c2) : R(0);
-    const R e2 = (DIM == 3) ? sel4(B2[2], c2) : R(0);
-    const R b12 = b1 * b2;
-    // the tap (c0, c1, c2) is b0 P + B1_0 Q + B2_0 T with the row's P, Q, T: the value,
-    // gradient and Laplacian weights factored along x
-    R Prow = vN * b12 + vG[1] * d1 * b2 + vL * (e1 * b2 + b1 * e2);
-    if (DIM == 3) Prow += vG[2] * b1 * d2;
-    const R Qrow = vG[0] * b12, Trow = vL * b12;
-    A* row = grad + (sel4i(o1, c1) + sel4i(o2, c2));
-#pragma unroll
-    for (int c0 = 0; c0 < 4; ++c0) {
-      const R val = B[0][c0] * Prow + B1[0][c0] * Qrow + B2[0][c0] * Trow;
-      if (val != R(0)) atomicAdd(&row[o0[c0]], A(val));
+  __syncwarp();
+  const AdjTap<R>* tx = st->tap + 33 * (lane & 3);
+  const AdjTap<R>* ty = st->tap + 33 * (4 + ((lane >> 2) & 3));
+  if (DIM == 3) {
+    const AdjTap<R>* tz = st->tap + 33 * (8 + (lane >> 4));
+    while (todo != 0u) {
+      const int e = __ffs(todo) - 1;
+      todo &= todo - 1u;
+      const AdjTap<R> X = tx[e], Y = ty[e], Z0 = tz[e], Z1 = tz[66 + e];
+      const R bb = X.b * Y.b, p = X.c * Y.b + X.b * Y.c;
+      A* row = grad + (X.off + Y.off);
+      const R v0 = Z0.b * p + Z0.c * bb, v1 = Z1.b * p + Z1.c * bb;
+      if (v0 != R(0)) atomicAdd(&row[Z0.off], A(v0));
+      if (v1 != R(0)) atomicAdd(&row[Z1.off], A(v1));
+    }
+  } else {
+    while (todo != 0u) {
+      const int e0 = __ffs(todo) - 1;
+      todo &= todo - 1u;
+      const int e1 = (todo != 0u) ? __ffs(todo) - 1 : -1;
+      todo &= todo - 1u;
+      const int e = (lane < 16) ? e0 : e1;
+      if (e >= 0) {
+        const AdjTap<R> X = tx[e], Y = ty[e];
+        const R val = X.c * Y.b + X.b * Y.c;
+        if (val != R(0)) atomicAdd(&grad[X.off + Y.off], A(val));
+      }
     }
   }
+  __syncwarp();
 }
 
 // d sigma' / d alpha_m = cN N_m + cG . grad N_m + cL Lap N_m at y, from the fields coeffs
@@ -179,30 +199,32 @@ __device__ void alpha_sensitivity(const FieldsAt<R>& F, R* cN, R* cG, R* cL) {
 // total and scatters.  The walks of one launch are items L.item_base .. + L.total_items.  Two
 // launches instead of one keep the lanes of a warp in one phase: in a single launch, lanes
 // whose walks were still in their first replay idled through the others' scatters.
-template <int DIM, typename R, bool ALPHA, int PASS>
+// MODE: what pass 2 scatters, ADJ_SIGMA or ADJ_ALPHA; the latter adds sigma's gradient from the same
+// replay when L.grad_sigma is set (both: 24.6 -> 14.8 ms where two calls replayed the walks four
+// times).  Pass 1 is the same for both.
+template <int DIM, typename R, int MODE, int PASS>
 __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) {
+  constexpr bool ALPHA = MODE == ADJ_ALPHA && PASS == 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   {
     const int4* src = reinterpret_cast<const int4*>(L.problem);
     int4* dst = reinterpret_cast<int4*>(smem_raw);
     for (int i = threadIdx.x; i < L.problem_bytes / 16; i += blockDim.x) dst[i] = src[i];
   }
-  // alpha: per-CTA accumulators in the walk's precision (FP32 shared atomics are native)
-  R* gpriv = reinterpret_cast<R*>(smem_raw + L.problem_bytes);
-  const bool priv = ALPHA && PASS == 2 && L.priv_nodes > 0;
+  // alpha: each warp's staged scatters, and the CTA's accumulators in the walk's precision (FP32
+  // shared atomics are native)
+  AdjStage<R>* stage = reinterpret_cast<AdjStage<R>*>(smem_raw + L.problem_bytes) + (threadIdx.x >> 5);
+  R* gpriv = reinterpret_cast<R*>(smem_raw + L.problem_bytes + (kAdjBlock / 32) * sizeof(AdjStage<R>));
+  const bool priv = ALPHA && L.priv_nodes > 0;
   R* totals = reinterpret_cast<R*>(L.totals);
   const DevProblem<R>& Pg0 = *reinterpret_cast<const DevProblem<R>*>(L.problem);
   const int64_t ares0 = Pg0.alpha.res[0], ares1 = Pg0.alpha.res[1];
-  const int64_t ps1 = ares0 + 1, ps2 = ps1 * ares1 + 1;  // padded shared layout
+  int64_t ps1 = 0, ps2 = 0;
+  adj_strides(ares0, ares1, &ps1, &ps2);
   if (priv)
     for (int i = threadIdx.x; i < L.priv_nodes; i += blockDim.x) gpriv[i] = R(0);
   __syncthreads();
   const DevProblem<R>& P = *reinterpret_cast<const DevProblem<R>*>(smem_raw);
-#define WOS_ALPHA_SCATTER(pt, a, b, c)                                                   \
-  do {                                                                                   \
-    if (priv) bspline_scatter<DIM, R, R>(P.alpha, pt, a, b, c, gpriv, ps1, ps2);         \
-    else bspline_scatter<DIM, R, double>(P.alpha, pt, a, b, c, L.grad_alpha, ares0, ares0 * ares1); \
-  } while (0)
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
   const R eps = R(L.eps), s_root = w_sqrt(R(L.sigma_bar));
@@ -267,14 +289,16 @@ __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) 
       need = __ballot_sync(0xffffffffu, !active);
     }
     if (__ballot_sync(0xffffffffu, active) == 0u) break;
-    if (!active) continue;
 
+    // alpha scatter of this iteration: vN N_m + vG . grad N_m + vL Lap N_m at y
+    R y[3] = {x[0], x[1], x[2]};
+    R vN = R(0), vG[3] = {R(0), R(0), R(0)}, vL = R(0);
+    if (active) {
     // pass 2 gives each walk one iteration of its own at x_0 first: the fields there give
     // e^{-gamma(x_0)} and the alpha term of x_0, which then goes through the same scatter
     // call as the steps' and the boundary's (lanes that start, step or end a walk in one
     // iteration scatter together instead of one after another)
     const bool first = (PASS == 2) && fresh;
-    R y[3] = {x[0], x[1], x[2]};
     R xb[3] = {R(0), R(0), R(0)};
     R d = R(0), dd = R(0), mu = R(1), Gn = R(0), PB = R(0);
     R dz[3] = {R(0), R(0), R(0)};
@@ -324,9 +348,7 @@ __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) 
     }
     R spy, fpy, gam, al;
     FieldsAt<R> fat;
-    coeffs<DIM, R, false>(P, y, &spy, &fpy, &gam, &al, nullptr, (ALPHA && PASS == 2) ? &fat : nullptr);
-    // alpha scatter of this iteration: vN N_m + vG . grad N_m + vL Lap N_m at y
-    R vN = R(0), vG[3] = {R(0), R(0), R(0)}, vL = R(0);
+    coeffs<DIM, R, false>(P, y, &spy, &fpy, &gam, &al, nullptr, ALPHA ? &fat : nullptr);
     if (first) {
       // grad_u e^{-gamma(x_0)} / walks; alpha: -A N_m(x_0) / (2 alpha(x_0))
       coef = R(__ldg(&L.grad_u[p]) * inv_walks) * w_exp(-gam);
@@ -338,7 +360,7 @@ __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) 
         const R bterm = W * w_exp(gam) * g_at<DIM>(P, xb);
         acc += bterm;
         // boundary factor e^{gamma(x_n)}: d/d alpha_m = N_m(x_n) / (2 alpha(x_n)) times the term
-        if (ALPHA && PASS == 2) vN = coef * bterm * R(0.5) / al;
+        if (ALPHA) vN = coef * bterm * R(0.5) / al;
       }
       if (PASS == 1) {
         totals[slot] = acc;  // the walk's total; the second pass replays it
@@ -351,7 +373,7 @@ __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) 
       const R src = W * Gn * fpy;
       acc += src;
       // source f'(y): d/d alpha_m = -N_m(y) / (2 alpha(y)) times the term
-      if (ALPHA && PASS == 2) vN = -coef * src * R(0.5) / al;
+      if (ALPHA) vN = -coef * src * R(0.5) / al;
       if (mu <= PB) {
         const R wj = R(1) - spy * inv_sb;
         if (PASS == 2) {
@@ -368,7 +390,8 @@ __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) 
               for (int i = 0; i < 3; ++i) vG[i] = rj * cG[i];
               vL = rj * cL;
             }
-          } else {
+          }
+          if (!ALPHA || L.grad_sigma != nullptr) {
             // d w_j / d sigma_m = -N_m(y) / (alpha(y) sigma_bar)
             const R val = -coef * rem * inv_sb / al;
             if (isfinite(val) && val != R(0)) grid_scatter<DIM, R>(P.sigma, y, val, L.grad_sigma);
@@ -384,7 +407,12 @@ __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) 
       if (PASS == 2) ++st_steps;
       ++k;
     }
-    if (ALPHA && PASS == 2 && isfinite(vN) && (vN != R(0) || vL != R(0))) WOS_ALPHA_SCATTER(y, vN, vG, vL);
+    }
+    if (ALPHA) {
+      const bool want = isfinite(vN) && (vN != R(0) || vL != R(0));
+      if (priv) bspline_scatter<DIM, R, R>(P.alpha, y, want, vN, vG, vL, gpriv, ps1, ps2, stage);
+      else bspline_scatter<DIM, R, double>(P.alpha, y, want, vN, vG, vL, L.grad_alpha, ares0, ares0 * ares1, stage);
+    }
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -393,9 +421,10 @@ __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) 
     st_capped += __shfl_down_sync(0xffffffffu, st_capped, off);
   }
   if (lane == 0 && L.stats != nullptr) {
-    atomicAdd(&L.stats[ST_STEPS], st_steps);
-    atomicAdd(&L.stats[ST_WALKS], (unsigned long long)st_walks);
-    if (st_capped) atomicAdd(&L.stats[ST_CAPPED], (unsigned long long)st_capped);
+    const unsigned long long each = (ALPHA && L.grad_sigma != nullptr) ? 2ull : 1ull;  // each gradient counts its replay
+    atomicAdd(&L.stats[ST_STEPS], each * st_steps);
+    atomicAdd(&L.stats[ST_WALKS], each * (unsigned long long)st_walks);
+    if (st_capped) atomicAdd(&L.stats[ST_CAPPED], each * (unsigned long long)st_capped);
   }
   if (priv) {
     __syncthreads();
@@ -406,21 +435,20 @@ __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) 
       if (v != R(0)) atomicAdd(&L.grad_alpha[i], (double)v);
     }
   }
-#undef WOS_ALPHA_SCATTER
 }
 
 #if !defined(__CUDACC_RTC__)
 // one pass (L.pass 1 or 2) of the adjoint; the caller zeroes the work counter before each
-template <int DIM, typename R, bool ALPHA, int PASS>
+template <int DIM, typename R, int MODE, int PASS>
 cudaError_t launch_adjoint_m(const AdjLaunch& L, int num_sms, cudaStream_t stream) {
-  size_t smem = (size_t)L.problem_bytes + ((ALPHA && PASS == 2) ? (size_t)L.priv_nodes * sizeof(R) : 0);
+  const size_t smem = adjoint_smem(L, (int)sizeof(R));
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(wos_adjoint_kernel<DIM, R, ALPHA, PASS>,
+    cudaError_t e = cudaFuncSetAttribute(wos_adjoint_kernel<DIM, R, MODE, PASS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wos_adjoint_kernel<DIM, R, ALPHA, PASS>,
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wos_adjoint_kernel<DIM, R, MODE, PASS>,
                                                                 kAdjBlock, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
@@ -429,17 +457,15 @@ cudaError_t launch_adjoint_m(const AdjLaunch& L, int num_sms, cudaStream_t strea
   if ((uint64_t)grid > blocks_needed) grid = (int)(blocks_needed > 0 ? blocks_needed : 1);
   AdjLaunch arg = L;
   philox_round_keys(arg.seed, arg.rk);
-  wos_adjoint_kernel<DIM, R, ALPHA, PASS><<<grid, kAdjBlock, smem, stream>>>(arg);
+  wos_adjoint_kernel<DIM, R, MODE, PASS><<<grid, kAdjBlock, smem, stream>>>(arg);
   return cudaGetLastError();
 }
 
 template <int DIM, typename R>
 cudaError_t launch_adjoint_t(const AdjLaunch& L, int num_sms, cudaStream_t stream) {
-  if (L.pass == 1)
-    return L.alpha ? launch_adjoint_m<DIM, R, true, 1>(L, num_sms, stream)
-                   : launch_adjoint_m<DIM, R, false, 1>(L, num_sms, stream);
-  return L.alpha ? launch_adjoint_m<DIM, R, true, 2>(L, num_sms, stream)
-                 : launch_adjoint_m<DIM, R, false, 2>(L, num_sms, stream);
+  if (L.pass == 1) return launch_adjoint_m<DIM, R, ADJ_SIGMA, 1>(L, num_sms, stream);
+  return L.mode == ADJ_ALPHA ? launch_adjoint_m<DIM, R, ADJ_ALPHA, 2>(L, num_sms, stream)
+                             : launch_adjoint_m<DIM, R, ADJ_SIGMA, 2>(L, num_sms, stream);
 }
 #endif  // !__CUDACC_RTC__
 

@@ -1086,7 +1086,7 @@ int wos_problem_specialized(const wos_problem* pr, int32_t* flags_out) {
     for (int v = 0; v < wos::kJitVariants; ++v)
       if (pr->jit.kernel[p][v] != nullptr) f |= (p ? WOS_SPEC_FP64 : WOS_SPEC_FP32) | vbit[v];
   for (int p = 0; p < 2; ++p)
-    if (pr->jit.adjoint[p][0][0] != nullptr) f |= (p ? WOS_SPEC_FP64 : WOS_SPEC_FP32) | WOS_SPEC_ADJOINT;
+    if (pr->jit.adjoint[p][0] != nullptr) f |= (p ? WOS_SPEC_FP64 : WOS_SPEC_FP32) | WOS_SPEC_ADJOINT;
   *flags_out = f;
   return WOS_OK;
 }
@@ -1215,7 +1215,7 @@ int adjoint_run(wos_ctx* ctx, const wos_problem* pr, wos::AdjLaunch& L, bool fp6
       L.pass = pass;
       cudaError_t e = cudaMemsetAsync(ctx->scratch, 0, sizeof(unsigned long long), st);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemsetAsync(work counter)");
-      cudaKernel_t spec = pr->jit.adjoint[fp64 ? 1 : 0][L.alpha ? 1 : 0][pass - 1];
+      cudaKernel_t spec = pr->jit.adjoint[fp64 ? 1 : 0][pass == 1 ? 0 : 1 + L.mode];
       if (spec != nullptr) e = wos::launch_adjoint_kernel(L, spec, (int)rb, ctx->num_sms, st);
       else e = fp64 ? wos::launch_adjoint_f64(L, ctx->num_sms, st) : wos::launch_adjoint_f32(L, ctx->num_sms, st);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "adjoint kernel launch");
@@ -1226,9 +1226,10 @@ int adjoint_run(wos_ctx* ctx, const wos_problem* pr, wos::AdjLaunch& L, bool fp6
 }
 }  // namespace
 
-extern "C" int wos_adjoint_sigma(wos_ctx* ctx, const wos_problem* pr, const float* pts, int64_t npts,
-                                 int32_t walks_uniform, const wos_params* prm, const double* grad_u,
-                                 double* grad_sigma, uint64_t* stats, void* stream) {
+// Adds the gradients whose arrays are not null (at least one), by one pair of passes.
+int adjoint_gradients(wos_ctx* ctx, const wos_problem* pr, const float* pts, int64_t npts, int32_t walks_uniform,
+                      const wos_params* prm, const double* grad_u, double* grad_sigma, double* grad_alpha,
+                      uint64_t* stats, void* stream) {
   if (!ctx) return WOS_EINVAL;
   if (!pr) return fail(ctx, WOS_EINVAL, "null problem");
   int rc = validate_params(ctx, prm);
@@ -1237,15 +1238,19 @@ extern "C" int wos_adjoint_sigma(wos_ctx* ctx, const wos_problem* pr, const floa
   if (npts < 0 || walks_uniform < 0) return fail(ctx, WOS_EINVAL, "negative size");
   if (npts > 0xffffffffll) return fail(ctx, WOS_EINVAL, "more than 2^32 points in one call");
   if (npts == 0 || walks_uniform == 0) return WOS_OK;
-  if (!pts || !grad_u || !grad_sigma) return fail(ctx, WOS_EINVAL, "null device array");
+  if (!pts || !grad_u || (!grad_sigma && !grad_alpha)) return fail(ctx, WOS_EINVAL, "null device array");
   const DevProblem<double>& H = pr->host64;
   if (H.has_drift) return fail(ctx, WOS_EUNSUPPORTED, "the adjoint has no extra-drift (omega) term");
-  if (H.sigma.kind != wos::F_GRID_LINEAR)
+  if (grad_sigma && H.sigma.kind != wos::F_GRID_LINEAR)
     return fail(ctx, WOS_EUNSUPPORTED, "the sigma gradient needs sigma given as a multilinear grid");
+  if (grad_alpha && H.alpha.kind != wos::F_GRID_BSPLINE)
+    return fail(ctx, WOS_EUNSUPPORTED, "the alpha gradient needs alpha given as a B-spline grid");
   if (H.f.kind == wos::F_MANUFACTURED)
-    return fail(ctx, WOS_EUNSUPPORTED, "a manufactured source depends on sigma; give f explicitly");
+    return fail(ctx, WOS_EUNSUPPORTED, std::string("a manufactured source depends on ") +
+                                           (grad_sigma ? "sigma" : "alpha") + "; give f explicitly");
   DeviceGuard g(ctx->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const bool fp64 = prm->precision == WOS_FP64;
   wos::AdjLaunch L;
   std::memset(&L, 0, sizeof(L));
   L.dim = pr->dim;
@@ -1260,9 +1265,29 @@ extern "C" int wos_adjoint_sigma(wos_ctx* ctx, const wos_problem* pr, const floa
   L.max_steps = prm->max_steps;
   L.grad_u = grad_u;
   L.grad_sigma = grad_sigma;
+  L.grad_alpha = grad_alpha;
+  L.mode = grad_alpha ? wos::ADJ_ALPHA : wos::ADJ_SIGMA;
   L.stats = reinterpret_cast<unsigned long long*>(stats);
   L.radial_tab = ctx->radial_tab[pr->dim - 2];
-  return adjoint_run(ctx, pr, L, prm->precision == WOS_FP64, st);
+  if (grad_alpha) {
+    // grids of up to 8192 nodes are accumulated per CTA in shared memory, where the padded copy fits
+    const int64_t planes = pr->dim == 3 ? H.alpha.res[2] : 1;
+    int64_t s1 = 0, s2 = 0;
+    wos::adj_strides(H.alpha.res[0], H.alpha.res[1], &s1, &s2);
+    if ((int64_t)H.alpha.res[0] * H.alpha.res[1] * planes <= 8192) {
+      L.priv_nodes = (int)(s2 * planes);
+      L.pass = 2;
+      L.problem_bytes = (int)(fp64 ? sizeof(DevProblem<double>) : sizeof(DevProblem<float>));
+      if (wos::adjoint_smem(L, fp64 ? 8 : 4) > 200 * 1024) L.priv_nodes = 0;
+    }
+  }
+  return adjoint_run(ctx, pr, L, fp64, st);
+}
+
+extern "C" int wos_adjoint_sigma(wos_ctx* ctx, const wos_problem* pr, const float* pts, int64_t npts,
+                                 int32_t walks_uniform, const wos_params* prm, const double* grad_u,
+                                 double* grad_sigma, uint64_t* stats, void* stream) {
+  return adjoint_gradients(ctx, pr, pts, npts, walks_uniform, prm, grad_u, grad_sigma, nullptr, stats, stream);
 }
 
 namespace wos {
@@ -1301,46 +1326,7 @@ extern "C" int wos_render_slice(wos_ctx* ctx, const wos_problem* pr, const wos_v
 extern "C" int wos_adjoint_alpha(wos_ctx* ctx, const wos_problem* pr, const float* pts, int64_t npts,
                                  int32_t walks_uniform, const wos_params* prm, const double* grad_u,
                                  double* grad_alpha, uint64_t* stats, void* stream) {
-  if (!ctx) return WOS_EINVAL;
-  if (!pr) return fail(ctx, WOS_EINVAL, "null problem");
-  int rc = validate_params(ctx, prm);
-  if (rc) return rc;
-  if ((rc = no_window(ctx, prm))) return rc;
-  if (npts < 0 || walks_uniform < 0) return fail(ctx, WOS_EINVAL, "negative size");
-  if (npts > 0xffffffffll) return fail(ctx, WOS_EINVAL, "more than 2^32 points in one call");
-  if (npts == 0 || walks_uniform == 0) return WOS_OK;
-  if (!pts || !grad_u || !grad_alpha) return fail(ctx, WOS_EINVAL, "null device array");
-  const DevProblem<double>& H = pr->host64;
-  if (H.has_drift) return fail(ctx, WOS_EUNSUPPORTED, "the adjoint has no extra-drift (omega) term");
-  if (H.alpha.kind != wos::F_GRID_BSPLINE)
-    return fail(ctx, WOS_EUNSUPPORTED, "the alpha gradient needs alpha given as a B-spline grid");
-  if (H.f.kind == wos::F_MANUFACTURED)
-    return fail(ctx, WOS_EUNSUPPORTED, "a manufactured source depends on alpha; give f explicitly");
-  int64_t nodes = (int64_t)H.alpha.res[0] * H.alpha.res[1] * (pr->dim == 3 ? H.alpha.res[2] : 1);
-  DeviceGuard g(ctx->device);
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  wos::AdjLaunch L;
-  std::memset(&L, 0, sizeof(L));
-  L.dim = pr->dim;
-  L.pts = pts;
-  L.npts = npts;
-  L.walks_uniform = walks_uniform;
-  L.total_items = (uint64_t)npts * (uint64_t)walks_uniform;
-  L.seed = prm->seed;
-  L.walk_offset = prm->walk_offset;
-  L.eps = prm->eps;
-  L.sigma_bar = prm->sigma_bar;
-  L.max_steps = prm->max_steps;
-  L.grad_u = grad_u;
-  L.grad_alpha = grad_alpha;
-  L.alpha = 1;
-  L.stats = reinterpret_cast<unsigned long long*>(stats);
-  L.radial_tab = ctx->radial_tab[pr->dim - 2];
-  // grids of up to 8192 nodes (64 KB of FP64) are accumulated per CTA in shared memory
-  // the per-CTA copy is padded (row stride res0 + 1, plane stride (res0 + 1) res1 + 1)
-  int64_t padded = ((int64_t)(H.alpha.res[0] + 1) * H.alpha.res[1] + 1) * (pr->dim == 3 ? H.alpha.res[2] : 1);
-  L.priv_nodes = (nodes <= 8192) ? (int)padded : 0;
-  return adjoint_run(ctx, pr, L, prm->precision == WOS_FP64, st);
+  return adjoint_gradients(ctx, pr, pts, npts, walks_uniform, prm, grad_u, nullptr, grad_alpha, stats, stream);
 }
 
 extern "C" int wos_batch_create(wos_ctx* ctx, const wos_problem* const* probs, int32_t nprob,

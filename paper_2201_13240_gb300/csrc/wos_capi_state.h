@@ -45,6 +45,12 @@ struct wos_ctx {
   size_t adj_totals_bytes = 0;
 };
 
+// wos_adjoint_sigma and wos_adjoint_alpha in one (wos_capi.cu): adds the gradients whose arrays are
+// not null
+int adjoint_gradients(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts, int32_t walks_uniform,
+                      const wos_params* params, const double* grad_u, double* grad_sigma, double* grad_alpha,
+                      uint64_t* stats, void* stream);
+
 struct wos_batch {
   wos_ctx* ctx = nullptr;
   int device = 0;                     // kept here: destroy must not read a destroyed context

@@ -479,11 +479,9 @@ int wos_adjoint(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t
   }
   cudaError_t e = cudaMemsetAsync(ctx->adj_buf, 0, sizeof(double) * (size_t)(ns + na), st);
   if (e != cudaSuccess) return hcuda(ctx, e, "zero gradient buffer");
-  int rc = WOS_OK;
-  if (grad_sigma)
-    rc = wos_adjoint_sigma(ctx, prob, pts, npts, walks_uniform, params, grad_u, ctx->adj_buf, stats, stream);
-  if (rc == WOS_OK && grad_alpha)
-    rc = wos_adjoint_alpha(ctx, prob, pts, npts, walks_uniform, params, grad_u, ctx->adj_buf + ns, stats, stream);
+  const int rc = adjoint_gradients(ctx, prob, pts, npts, walks_uniform, params, grad_u,
+                                   grad_sigma ? ctx->adj_buf : nullptr, grad_alpha ? ctx->adj_buf + ns : nullptr,
+                                   stats, stream);
   if (rc != WOS_OK) return rc;
   if (grad_sigma) to_float_kernel<<<grid_blocks(ctx, ns), 256, 0, st>>>(ctx->adj_buf, ns, grad_sigma);
   if (grad_alpha) to_float_kernel<<<grid_blocks(ctx, na), 256, 0, st>>>(ctx->adj_buf + ns, na, grad_alpha);

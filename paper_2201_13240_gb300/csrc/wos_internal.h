@@ -79,6 +79,19 @@ struct WalkLaunch {
   uint32_t rk[20];
 };
 
+enum { ADJ_SIGMA = 0, ADJ_ALPHA = 1 };
+// The per-CTA copy of an alpha grid in shared memory: strides of its rows and planes.  The 32 taps a
+// warp adds at once are 4 x 4 x 2 neighbours; with a row stride of 4 (mod 8) and a plane stride of
+// 16 (mod 32) they lie in 32 different banks.
+#if defined(__CUDACC__)
+__host__ __device__
+#endif
+inline void adj_strides(int64_t res0, int64_t res1, int64_t* s1, int64_t* s2) {
+  *s1 = res0 + (12 - res0 % 8) % 8;
+  const int64_t plane = *s1 * res1;
+  *s2 = plane + (48 - plane % 32) % 32;
+}
+
 // adjoint launch: d(sum_p grad_u[p] mean_u[p]) / d(sigma grid nodes), added to grad_sigma
 struct AdjLaunch {
   const void* problem;
@@ -95,9 +108,9 @@ struct AdjLaunch {
   double sigma_bar;
   int64_t max_steps;
   const double* grad_u;           // [npts]
-  double* grad_sigma;             // [sigma grid nodes], accumulated (sigma launches)
+  double* grad_sigma;             // [sigma grid nodes], accumulated, or null
   double* grad_alpha;             // [alpha grid nodes], accumulated (alpha launches)
-  int alpha;                      // 1: gradient with respect to the alpha B-spline grid
+  int mode;                       // ADJ_SIGMA, or ADJ_ALPHA (with sigma's gradient too if grad_sigma is set)
   int priv_nodes;                 // > 0: accumulate per CTA in shared memory over this many nodes
   unsigned long long* stats;      // optional
   unsigned long long* work_counter;
@@ -108,6 +121,8 @@ struct AdjLaunch {
 };
 
 #if !defined(__CUDACC_RTC__)
+// shared memory of an adjoint launch; real_bytes: the walk's precision
+size_t adjoint_smem(const AdjLaunch& L, int real_bytes);
 cudaError_t launch_adjoint_f32(const AdjLaunch& L, int num_sms, cudaStream_t stream);
 cudaError_t launch_adjoint_f64(const AdjLaunch& L, int num_sms, cudaStream_t stream);
 // an adjoint kernel compiled at run time for one problem (same parameter block and launch shape)

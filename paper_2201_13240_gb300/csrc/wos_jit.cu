@@ -472,14 +472,13 @@ int jit_compile(const DevProblem<double>& P, bool fp64, int variant_mask, std::v
     *log = std::string("nvrtcCreateProgram: ") + api.GetErrorString(r);
     return WOS_EUNSUPPORTED;
   }
-  // walk variants at 0..kJitVariants-1, then the adjoint kernels (sigma pass 1, 2, alpha pass 1, 2)
+  // walk variants at 0..kJitVariants-1, then the adjoint kernels (pass 1; pass 2 by mode)
   std::vector<std::string> exprs(kJitExprs);
   if (variant_mask & (1 << kJitAdjoint)) {
-    const std::string t = std::to_string(P.dim) + ", " + (fp64 ? "double" : "float");
-    for (int a = 0; a < 2; ++a)
-      for (int pass = 1; pass <= 2; ++pass)
-        exprs[kJitVariants + 2 * a + pass - 1] = "wos::wos_adjoint_spec_kernel<" + t + (a ? ", true, " : ", false, ") +
-                                                 std::to_string(pass) + ">";
+    const std::string t = "wos::wos_adjoint_spec_kernel<" + std::to_string(P.dim) + ", " + (fp64 ? "double" : "float") +
+                          ", ";
+    exprs[kJitVariants] = t + "0, 1>";
+    for (int mode = 0; mode < 2; ++mode) exprs[kJitVariants + 1 + mode] = t + std::to_string(mode) + ", 2>";
   }
   for (int v = 0; v < kJitExprs; ++v) {
     if (v < kJitVariants) {
@@ -536,7 +535,7 @@ int jit_specialise(JitState* js, const DevProblem<double>& P, bool fp64, int var
   int need = 0;
   for (int v = 0; v < kJitVariants; ++v)
     if ((variant_mask & (1 << v)) && js->kernel[p][v] == nullptr) need |= 1 << v;
-  if ((variant_mask & (1 << kJitAdjoint)) && js->adjoint[p][0][0] == nullptr) need |= 1 << kJitAdjoint;
+  if ((variant_mask & (1 << kJitAdjoint)) && js->adjoint[p][0] == nullptr) need |= 1 << kJitAdjoint;
   if (need == 0) return WOS_OK;
   std::vector<char> cubin;
   std::vector<std::string> lowered;
@@ -569,8 +568,7 @@ int jit_specialise(JitState* js, const DevProblem<double>& P, bool fp64, int var
   for (int v = 0; v < kJitVariants; ++v)
     if (need & (1 << v)) js->kernel[p][v] = found[v];
   if (need & (1 << kJitAdjoint)) {
-    for (int a = 0; a < 2; ++a)
-      for (int q = 0; q < 2; ++q) js->adjoint[p][a][q] = found[kJitVariants + 2 * a + q];
+    for (int k = 0; k < 3; ++k) js->adjoint[p][k] = found[kJitVariants + k];
   }
   js->libs.push_back(lib);
   return WOS_OK;
@@ -581,9 +579,8 @@ void jit_release(JitState* js) {
   js->libs.clear();
   for (auto& row : js->kernel)
     for (auto& k : row) k = nullptr;
-  for (auto& plane : js->adjoint)
-    for (auto& row : plane)
-      for (auto& k : row) k = nullptr;
+  for (auto& row : js->adjoint)
+    for (auto& k : row) k = nullptr;
 }
 
 }  // namespace wos

@@ -11,13 +11,13 @@
 namespace wos {
 
 // kernel variants of one problem and precision (the domain fixes MESH, the problem DRIFT);
-// bit kJitAdjoint of a variant mask asks for the path-replay adjoint kernels (sigma and alpha,
-// each as its two passes); kJitExprs counts the kernels one program can hold
-enum { kJitPlain = 0, kJitWindow = 1, kJitGrad = 2, kJitVariants = 3, kJitAdjoint = 3, kJitExprs = 7 };
+// bit kJitAdjoint of a variant mask asks for the path-replay adjoint kernels (pass 1, and pass 2 for
+// sigma and for alpha); kJitExprs counts the kernels one program can hold
+enum { kJitPlain = 0, kJitWindow = 1, kJitGrad = 2, kJitVariants = 3, kJitAdjoint = 3, kJitExprs = 6 };
 
 struct JitState {
   cudaKernel_t kernel[2][kJitVariants] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};  // [fp64]
-  cudaKernel_t adjoint[2][2][2] = {};  // [fp64][alpha][pass - 1]
+  cudaKernel_t adjoint[2][3] = {};  // [fp64][0: pass 1, 1 + mode: pass 2]
   std::vector<cudaLibrary_t> libs;
 };
 
