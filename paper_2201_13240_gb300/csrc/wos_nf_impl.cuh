@@ -37,8 +37,12 @@ namespace wos {
 constexpr int kNfBlock = 128;
 constexpr uint64_t kNfChunk = 128;
 
+// Resident blocks per SM: series 4 / 5 / 6 measured 21.6 / 20.7 / 21.1 ms, printed approximations 12.4 /
+// 11.9 / 10.9 ms (32^3 points x 96 walks of the 3D workload).  The kernel is bound by its code's size (a
+// third of its stalls waited for instructions) and by the sweeps' arithmetic: the sweep split at the
+// last term, its loops rolled, and divisions by known integers took the series from 28.2 to 20.7 ms.
 template <int DIM, typename R, bool MESH, bool SERIES>
-__global__ void __launch_bounds__(kNfBlock, (sizeof(R) == 4) ? 4 : 1) wos_nf_kernel(WalkLaunch L) {
+__global__ void __launch_bounds__(kNfBlock, (sizeof(R) == 4) ? (SERIES ? 5 : 6) : 1) wos_nf_kernel(WalkLaunch L) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   {
     const int4* src = reinterpret_cast<const int4*>(L.problem);
