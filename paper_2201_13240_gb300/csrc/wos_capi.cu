@@ -409,6 +409,19 @@ int no_window(wos_ctx* ctx, const wos_params* prm) {
   return WOS_OK;
 }
 
+// The register cap of the generic FP32 value kernel (five blocks per SM otherwise).  3D B-spline
+// fields keep 64 taps' weights and indices: four blocks (a noise cube, 4096 points x 256 walks: 4 / 5 /
+// 6 / 8 blocks 4.21 / 4.70 / 5.38 / 5.94 ms; in 2D 4.77 / 4.51 / 4.46 / 4.81).  Closed-form fields keep
+// little and wait on the interpreter's chains: eight, where there are walks enough to fill them
+// (2D square 8.4e6 walks 6.24 / 5.58 / 5.27 / 5.07 ms, 3D cube 4.2e6 walks 8.77 / 7.91 / 7.46 / 7.21; a
+// solve of 2.6e5 walks 441 / 437 / 450 / 495 us).
+int generic_variant(const DevProblem<double>& P, uint64_t total) {
+  const wos::DevField<double>* fields[6] = {&P.alpha, &P.phi, &P.sigma, &P.f, &P.g, &P.um};
+  for (const wos::DevField<double>* f : fields)
+    if (f->kind == wos::F_GRID_BSPLINE) return P.dim == 3 ? 2 : 0;
+  return total > wos::kSpreadItems ? 1 : 0;
+}
+
 int launch(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts, const int64_t* walk_end,
            int64_t walks_uniform, uint64_t total, const wos_params* prm, double* sum, double* sumsq,
            int64_t* count, uint64_t* stats, double* uhat, int64_t* steps, cudaStream_t st,
@@ -476,6 +489,7 @@ int launch(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts
   } else {
     L.problem = prob->d32;
     L.problem_bytes = (int)sizeof(DevProblem<float>);
+    L.regs_variant = generic_variant(prob->host64, walk_end ? ~0ull : total);
     e = nf ? wos::launch_nf_f32(L, ctx->num_sms, st) : wos::launch_walks_f32(L, ctx->num_sms, st);
   }
   if (e == cudaSuccess && spread) e = wos::launch_walk_sums(L, L.ww_lo == 0.0 && !L.mesh, st);

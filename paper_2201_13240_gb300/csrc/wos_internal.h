@@ -63,7 +63,8 @@ struct WalkLaunch {
   int32_t nf_series;
   int drift;                      // the problem has an extra drift (omega fields)
   // launch schedule (0 = the kernel's own rule): walks claimed per warp at a time, resident
-  // blocks launched per SM, and the register-cap variant of batched launches (1: 8 blocks/SM)
+  // blocks launched per SM, and the register-cap variant of batched and generic FP32 value launches
+  // (1: 8 blocks/SM, 2, not batched: 4)
   uint32_t chunk;
   int32_t blocks_per_sm;
   int32_t regs_variant;

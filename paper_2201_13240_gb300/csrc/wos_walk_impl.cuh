@@ -184,8 +184,8 @@ constexpr int kMeshLeaves = 5;
 #else
 #define WOS_WALK_KERNEL wos_walk_kernel
 #endif
-// MINB > 0 overrides the resident-block target (the batched launches' high-occupancy
-// variant, chosen by the schedule).
+// MINB > 0 overrides the resident-block target (the batched launches' high-occupancy variant, chosen by
+// the schedule, and the value kernel's variants by fields and size, see generic_variant).
 template <int DIM, typename R, bool MESH, bool BATCHED, bool WW, bool GRAD, bool DRIFT = false, int MINB = 0>
 __global__ void __launch_bounds__(kWalkBlock,
                                   (sizeof(R) == 4) ? (GRAD ? 5 : (MESH ? kMeshBlocks : (MINB > 0 ? MINB : WOS_WALK_MIN_BLOCKS))) : 1)
@@ -778,6 +778,9 @@ cudaError_t launch_walks_t(const WalkLaunch& L, int num_sms, cudaStream_t stream
     return (DIM == 3 && L.mesh) ? launch_walks_m<DIM, R, true, false, false, true>(L, num_sms, stream)
                                 : launch_walks_m<DIM, R, false, false, false, true>(L, num_sms, stream);
   const bool ww = L.ww_lo > 0.0;
+  if (sizeof(R) == 4 && !ww && !L.mesh && L.regs_variant != 0)
+    return (L.regs_variant == 1) ? launch_walks_m<DIM, R, false, false, false, false, false, 8>(L, num_sms, stream)
+                                 : launch_walks_m<DIM, R, false, false, false, false, false, 4>(L, num_sms, stream);
   if (DIM == 3 && L.mesh)
     return ww ? launch_walks_m<DIM, R, true, false, true>(L, num_sms, stream)
               : launch_walks_m<DIM, R, true, false, false>(L, num_sms, stream);

@@ -64,3 +64,23 @@ def test_per_point_counts(most):
     u = torch.where(torch.arange(most, device="cuda")[None, :] < torch.from_numpy(counts).cuda()[:, None], u, 0.0)
     tol = max(128, most) * 2.0 ** -24
     assert torch.all((s - u.sum(1)).abs() <= tol * u.abs().sum(1))
+
+
+@pytest.mark.parametrize("kind", ["square2d", "cube3d", "noise_cube", "noise_annulus"])
+def test_register_variants_walk_the_same_walks(kind):
+    """The generic kernel's variants (by fields, and above 2^20 walks) run the same arithmetic."""
+    import torch
+    ctx = _ctx()
+    desc = {"square2d": W.square2d_problem, "cube3d": W.cube3d_problem, "noise_cube": W.noise_cube_problem,
+            "noise_annulus": W.noise_annulus_problem}[kind]()
+    prob = ctx.problem(desc)
+    rng = np.random.default_rng(1)
+    n = 64
+    r, t = np.sqrt(rng.uniform(0.4 ** 2, 1.05 ** 2, n)), rng.uniform(0, 2 * np.pi, n)
+    pts = np.stack([r * np.cos(t), r * np.sin(t)]).astype(np.float32) if kind == "noise_annulus" else \
+        W.uniform_in_box(desc["dim"], n, 0.05, 0.95, 2)
+    pts = torch.from_numpy(pts).cuda()
+    many = (1 << 20) // n + 1
+    a, ka, _ = ctx.walk_estimates(prob, pts, 50, 1e-3, 40.0, seed=3)
+    b, kb, _ = ctx.walk_estimates(prob, pts, many, 1e-3, 40.0, seed=3)
+    assert torch.equal(a, b[:, :50]) and torch.equal(ka, kb[:, :50])
