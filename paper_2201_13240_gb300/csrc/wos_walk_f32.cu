@@ -32,6 +32,11 @@ cudaError_t launch_walks_kernel(const WalkLaunch& L, cudaKernel_t kernel, int re
   return cudaLaunchKernel(fn, dim3(grid), dim3(kWalkBlock), args, smem, stream);
 }
 
+struct SumRun {
+  uint32_t p, n;        // point, walks
+  float sh, d1, d2;     // the first walk's value, and the sums of differences from it and of their squares
+};
+
 // Per-point sums of a small solve from its walks' totals (item_acc, in item order).
 //
 // What bounds it: nothing much (12 bytes per walk, ~25 rounds of a warp per 128 walks); it exists
@@ -43,7 +48,7 @@ cudaError_t launch_walks_kernel(const WalkLaunch& L, cudaKernel_t kernel, int re
 // The order of the sums is the persistent kernel's: FP32 partial sums per lane, shifted by the
 // lane's first walk of the point, over the walks that lane would have run had one warp taken
 // 128 consecutive walks, each lane that is free claiming the next one (lanes free at the same
-// iteration in lane order, GATHERED: once kDeferLanes lanes are free).  A solve's sums therefore
+// iteration in lane order, GATHERED: once four lanes are free).  A solve's sums therefore
 // do not depend on which warp ran which walk, and equal those of larger chunks' launches.
 template <bool GATHERED>
 __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__ acc, const uint32_t* __restrict__ iters,
@@ -66,38 +71,35 @@ __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__
     a[q] = in ? acc[base + 32 * q + lane] : 0.0f;
     it[q] = in ? iters[base + 32 * q + lane] : 0u;
   }
-  uint32_t p = 0xffffffffu, n_acc = 0;
-  float sh = 0.0f, d1 = 0.0f, d2 = 0.0f;
-  auto flush = [&]() {
-    if (n_acc == 0u) return;
-    const double e0 = (double)scale[p], c = (double)sh, m = (double)n_acc;
-    const double s1 = m * c + (double)d1, s2 = m * c * c + 2.0 * c * (double)d1 + (double)d2;
-    atomicAdd(&sum[p], s1 * e0);
-    atomicAdd(&sumsq[p], s2 * e0 * e0);
-    atomicAdd(&count[p], (unsigned long long)n_acc);
+  // A lane's sums over consecutive walks of one point are a run; runs wait in shared memory until the
+  // walks are through, so that their FP64 arithmetic is done by all lanes at once, and runs of one
+  // point meet in one atomic (flushed as they end, by a lane or two: 2.6e5 points x 4 walks of the 3D
+  // cube 808 us, so 680; 30 points x 8192 walks 386 us, so 299).
+  __shared__ SumRun runs[4][kChunkMin];
+  SumRun* run = runs[threadIdx.x >> 5];
+  uint32_t n_runs = 0;  // of the warp
+  SumRun r = {0xffffffffu, 0u, 0.0f, 0.0f, 0.0f};
+  auto add = [&](bool on, uint32_t item, float v) {
+    const uint32_t q = on ? point[item] : r.p;
+    const bool ends = on && r.n != 0u && q != r.p;
+    const unsigned done = __ballot_sync(kFull, ends);
+    if (ends) run[n_runs + __popc(done & ((1u << lane) - 1u))] = r;
+    n_runs += __popc(done);
+    if (!on) return;
+    if (q != r.p) r = SumRun{q, 0u, v, 0.0f, 0.0f};
+    const float dv = v - r.sh;
+    r.d1 += dv;
+    r.d2 += dv * dv;
+    ++r.n;
   };
-  auto add = [&](uint32_t item, float v) {
-    const uint32_t q = point[item];
-    if (q != p) {
-      flush();
-      p = q;
-      n_acc = 0;
-      sh = v;
-      d1 = d2 = 0.0f;
-    }
-    const float dv = v - sh;
-    d1 += dv;
-    d2 += dv * dv;
-    ++n_acc;
-  };
-  if (lane < n) add(base + lane, a[0]);
+  add(lane < n, base + lane, a[0]);
   uint32_t free_at = it[0];  // iteration at which the lane has no walk
   for (uint32_t next = 32; next < n;) {
     // the iteration of the next claim
     uint32_t t = __reduce_min_sync(kFull, free_at);
     if (GATHERED) {
       uint32_t rest = free_at;
-      for (int got = __popc(__ballot_sync(kFull, rest == t)); got < kDeferLanes;) {
+      for (int got = __popc(__ballot_sync(kFull, rest == t)); got < 4;) {
         if (rest == t) rest = 0xffffffffu;
         t = __reduce_min_sync(kFull, rest);
         got += __popc(__ballot_sync(kFull, rest == t));
@@ -116,13 +118,45 @@ __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__
         k = kq;
       }
     }
-    if ((claim >> lane & 1u) && j < n) {
-      add(base + j, v);
-      free_at = t + k;
-    }
+    const bool takes = (claim >> lane & 1u) && j < n;
+    add(takes, base + j, v);
+    if (takes) free_at = t + k;
     next += __popc(claim);
   }
-  flush();
+  const unsigned last = __ballot_sync(kFull, r.n != 0u);
+  if (r.n != 0u) run[n_runs + __popc(last & ((1u << lane) - 1u))] = r;
+  n_runs += __popc(last);
+  __syncwarp();
+  for (uint32_t at = 0; at < n_runs; at += 32) {
+    const bool on = at + lane < n_runs;
+    double s1 = 0.0, s2 = 0.0;
+    uint32_t m = 0, p = run[at].p;
+    if (on) {
+      const SumRun q = run[at + lane];
+      const double e0 = (double)scale[q.p], c = (double)q.sh, w = (double)q.n;
+      s1 = w * c + (double)q.d1;
+      s2 = w * c * c + 2.0 * c * (double)q.d1 + (double)q.d2;
+      s1 = s1 * e0;
+      s2 = s2 * e0 * e0;
+      m = q.n;
+      p = q.p;
+    }
+    // many walks per point: the warp's runs are of one point as a rule, and meet in one atomic each
+    const bool one = __all_sync(kFull, p == __shfl_sync(kFull, p, 0));
+    if (one) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        s1 += __shfl_down_sync(kFull, s1, off);
+        s2 += __shfl_down_sync(kFull, s2, off);
+        m += __shfl_down_sync(kFull, m, off);
+      }
+    }
+    if (one ? lane == 0 : on) {
+      atomicAdd(&sum[p], s1);
+      atomicAdd(&sumsq[p], s2);
+      atomicAdd(&count[p], (unsigned long long)m);
+    }
+  }
 }
 
 cudaError_t launch_walk_sums(const WalkLaunch& L, bool gathered, cudaStream_t stream) {
