@@ -140,7 +140,7 @@ cudaError_t launch_walks_kernel(const WalkLaunch& L, cudaKernel_t kernel, int re
                                 cudaStream_t stream);
 
 // adds the walks of a launch with per-walk buffers to L.sum, L.sumsq and L.count; `gathered`:
-// the walk kernel's lanes wait for each other's ends (kDeferLanes)
+// the walk kernel's lanes wait for each other's ends
 cudaError_t launch_walk_sums(const WalkLaunch& L, bool gathered, cudaStream_t stream);
 // per-walk buffers of a context in `buf` (4 * kSpreadItems words) for a launch that may take them
 inline void use_spread(WalkLaunch* L, float* buf) {

@@ -250,11 +250,15 @@ std::string kernel_expr(int dim, bool fp64, bool mesh, bool drift, int variant) 
 // 16^3 and 33^3 grids) 4.27 / 4.19 / 4.67 / 5.48 / 5.90 and 5.98 / 6.19 / 6.66 / 7.61 / 8.06 ms;
 // 2D (49^2 grids, 4096 x 1024) 3.32 / 3.06 / 3.01 / 3.15 / 3.25 ms and at 8 blocks 3.42 ms; a
 // batch of 192 2D problems 117.6 / 107.9 / 106.5 / 110.0 / 111.5 ms and at 8 blocks 117.4 ms.
-int min_blocks(const DevProblem<double>& P, bool batch) {
+// Gathered walk ends: see WOS_WALK_DEFER_LANES.
+std::string tuning(const DevProblem<double>& P, bool batch) {
   const DevField<double>* fields[6] = {&P.alpha, &P.phi, &P.sigma, &P.f, &P.g, &P.um};
-  for (const DevField<double>* f : fields)
-    if (f->kind == F_GRID_BSPLINE) return P.dim == 3 ? 4 : 5;
-  return P.dim == 3 ? (batch ? 7 : 6) : 8;
+  bool bspline = false;
+  for (const DevField<double>* f : fields) bspline = bspline || f->kind == F_GRID_BSPLINE;
+  const int blocks = bspline ? (P.dim == 3 ? 4 : 5) : (P.dim == 3 ? (batch ? 7 : 6) : 8);
+  const int gather = bspline ? 8 : (P.dim == 3 ? 4 : 6);
+  return "#define WOS_WALK_MIN_BLOCKS " + std::to_string(blocks) + "\n#define WOS_WALK_DEFER_LANES " +
+         std::to_string(gather) + "\n";
 }
 
 }  // namespace
@@ -274,8 +278,8 @@ std::string jit_source(const DevProblem<double>& P) {
     for (int i = 0; i < 16; ++i) s += (i ? ", " : "") + lit(P.dom[i]);
     s += "}\n";
   }
-  s += "#define WOS_WALK_MIN_BLOCKS " + std::to_string(min_blocks(P, false)) + "\n";
-  s += "#include \"wos_walk_impl.cuh\"\n#include \"wos_adjoint_impl.cuh\"\n\nnamespace wos {\n\n";
+  s += tuning(P, false);
+  s += "#include \"wos_walk_impl.cuh\"\n#if !defined(WOS_JIT_NO_ADJOINT)\n#include \"wos_adjoint_impl.cuh\"\n#endif\n\nnamespace wos {\n\n";
   s += "template <int DIM, typename R>\n";
   s += "__device__ __forceinline__ FieldVal<R> jit_field(const DevProblem<R>& P, int id, R x0, R x1, R x2, "
        "bool deriv) {\n";
@@ -318,7 +322,7 @@ std::string jit_source_batch(const BatchJitInfo& info) {
        "D): fields shared by every problem are generated code, the others are interpreted\n";
   s += "#define WOS_JIT_FIELDS 1\n";
   s += "#define WOS_JIT_F_KIND " + std::to_string(P.f.kind) + "\n";
-  s += "#define WOS_WALK_MIN_BLOCKS " + std::to_string(min_blocks(P, true)) + "\n";
+  s += tuning(P, true);
   s += "#include \"wos_walk_impl.cuh\"\n\nnamespace wos {\n\n";
   s += "template <int DIM, typename R>\n";
   s += "__device__ __forceinline__ FieldVal<R> jit_field(const DevProblem<R>& P, int id, R x0, R x1, R x2, "
@@ -494,8 +498,9 @@ int jit_compile(const DevProblem<double>& P, bool fp64, int variant_mask, std::v
       return WOS_EUNSUPPORTED;
     }
   }
-  const char* opts[] = {"-arch=sm_103a", "-std=c++17", "-lineinfo"};
-  r = api.CompileProgram(prog, 3, opts);
+  // the adjoint's header is parsed only for programs that hold its kernels
+  const char* opts[] = {"-arch=sm_103a", "-std=c++17", "-lineinfo", "-DWOS_JIT_NO_ADJOINT"};
+  r = api.CompileProgram(prog, (variant_mask & (1 << kJitAdjoint)) ? 3 : 4, opts);
   size_t ls = 0;
   api.GetProgramLogSize(prog, &ls);
   std::string plog(ls, '\0');

@@ -60,11 +60,17 @@ struct WalkState {
 };
 
 constexpr int kWWDepth = 8;  // most split copies a lane keeps waiting
+// Ended walks a warp gathers before finishing them: the end and the regeneration run for those
+// lanes together, while the waiting ones sit out a few steps.  The costlier a step, the later: the
+// generated source sets it by the problem's fields, gradient walks (whose ends are the costliest) take
+// eight.  Measured at 4 / 6 / 8 / 10 / 12 lanes: gradient 9.95 / 9.40 / 9.21 / 9.19 / 9.29 ms (32^3 points
+// x 512 walks), a batch 47.9 / 46.6 / 46.2 / 46.2 / 46.5 (96 problems), 3D B-spline fields 7.98 / 7.77 /
+// 7.63 / 7.59 / 7.65 (4.2e6 walks), the 2D square 4.52 / 4.48 and 4.49 at 8 (1.7e7 walks), the 3D cube
+// 28.69 / 28.78 and 29.28 at 8 (6.7e7 walks).
 #if !defined(WOS_WALK_DEFER_LANES)
 #define WOS_WALK_DEFER_LANES 4
 #endif
-constexpr int kDeferLanes = WOS_WALK_DEFER_LANES;  // ended walks a warp gathers before finishing them
-static_assert(kDeferLanes >= 1 && kDeferLanes <= 32, "kDeferLanes must be 1..32");
+static_assert(WOS_WALK_DEFER_LANES >= 1 && WOS_WALK_DEFER_LANES <= 32, "1..32 lanes");
 
 // e^{-gamma(x_0)} of point p (applied once per flush), in the walk's precision: the
 // FP32 walk's gamma carries FP32 rounding already, and an FP64 exp costs dozens of
@@ -241,6 +247,11 @@ __global__ void __launch_bounds__(kWalkBlock,
   double s1 = 0.0, s2 = 0.0;
   uint32_t n_acc = 0;
   R sh = R(0), d1 = R(0), d2 = R(0);  // FP32 partial sums shifted by the point's first value
+  // SUM64: s1 and s2 are the sums themselves.  Where six or eight ends are finished at a time two FP64
+  // additions a walk cost less than the shift (a batch 46.2 -> 45.3 ms, the 2D square 4.48 -> 4.37; at four
+  // the 3D cube 109.8 -> 110.2 ms), and the shifted FP32 sums lose digits when a
+  // point's first walk is an outlier of a heavy-tailed estimate.
+  constexpr bool SUM64 = GRAD || WOS_WALK_DEFER_LANES >= 6;
   // spatial gradient: per-lane partial sums of (grad U - U grad gamma) and grad gamma(x_0)
   double gs1[3] = {0.0, 0.0, 0.0}, gs2[3] = {0.0, 0.0, 0.0};
   R ggam[3] = {R(0), R(0), R(0)};
@@ -263,6 +274,14 @@ __global__ void __launch_bounds__(kWalkBlock,
   const int ww_depth = WW ? (L.ww_depth < kWWDepth ? L.ww_depth : kWWDepth) : 0;
   const R ww_lo = R(L.ww_lo), ww_hi = R(L.ww_hi);
 
+  // the item of the lane's walk, for the per-walk outputs: carried (two registers), or found again from
+  // its point and walk id where the fields need the registers
+  auto item_of = [&]() -> uint64_t {
+    if (WOS_WALK_DEFER_LANES < 8) return s.item;
+    const uint64_t j = (uint64_t)(uint32_t)(s.w - (uint32_t)L.walk_offset);
+    if (L.walk_end == nullptr) return (uint64_t)s.p * (uint64_t)L.walks_uniform + j;
+    return (s.p > 0u ? (uint64_t)__ldg(&L.walk_end[s.p - 1u]) : 0ull) + j;
+  };
   // a walk's end once g is added: the spatial gradient, the per-point partial sums (flushed
   // when the lane moves to another point), the per-walk outputs and the statistics
   auto finish_walk = [&](const DevProblem<R>& Pw, bool capped) {
@@ -280,15 +299,10 @@ __global__ void __launch_bounds__(kWalkBlock,
 #pragma unroll
       for (int i = 0; i < DIM; ++i) gv[i] = (s.k == 0) ? R(NAN) : s.acc * (s.gb[i] - ggam[i]) + s.gc[i];
     }
-    if (spread) {
-      L.item_acc[s.item] = (float)s.acc;
-      L.item_point[s.item] = s.p;
-      L.item_iters[s.item] = WW ? s.steps_walk + s.next_bid : s.k + 1u;  // steps and branch ends
-      if (s.w == (uint32_t)L.walk_offset) L.point_scale[s.p] = (float)point_factor<DIM, R>(L, Pw, s.p);
-    } else if (accumulate && s.p != acc_p) {
+    if (!spread && accumulate && s.p != acc_p) {
       if (acc_p != kNoPoint) {
         double e0 = point_factor<DIM, R>(L, BATCHED ? Pall[acc_prob] : *Pshared, acc_p);
-        if (!GRAD) {
+        if (!SUM64) {
           double c = (double)sh, n = (double)n_acc;
           s1 = n * c + (double)d1;
           s2 = n * c * c + 2.0 * c * (double)d1 + (double)d2;
@@ -315,7 +329,7 @@ __global__ void __launch_bounds__(kWalkBlock,
       d1 = R(0);
       d2 = R(0);
     }
-    if (GRAD) {
+    if (SUM64) {
       const double acc_d = (double)s.acc;
       s1 += acc_d;
       s2 += acc_d * acc_d;
@@ -332,13 +346,26 @@ __global__ void __launch_bounds__(kWalkBlock,
         gs2[i] += (double)gv[i] * (double)gv[i];
       }
     }
-    if (L.uhat != nullptr) {
-      double e0 = point_factor<DIM, R>(L, Pw, s.p);
-      L.uhat[s.item] = (double)s.acc * e0;
-      L.steps_out[s.item] = WW ? (int64_t)s.steps_walk : (int64_t)s.k;
-      if (GRAD && L.ghat != nullptr) {
+    // per-walk outputs: a small solve's sums and its points' factors, or the caller's estimates
+    if (spread || L.uhat != nullptr) {
+      const uint64_t item = item_of();
+      if (spread) {
+        L.item_acc[item] = (float)s.acc;
+        L.item_point[item] = s.p;
+        L.item_iters[item] = WW ? s.steps_walk + s.next_bid : s.k + 1u;  // steps and branch ends
+      }
+      if (!spread || s.w == (uint32_t)L.walk_offset) {
+        const double e0 = point_factor<DIM, R>(L, Pw, s.p);
+        if (spread) {
+          L.point_scale[s.p] = (float)e0;
+        } else {
+          L.uhat[item] = (double)s.acc * e0;
+          L.steps_out[item] = WW ? (int64_t)s.steps_walk : (int64_t)s.k;
+          if (GRAD && L.ghat != nullptr) {
 #pragma unroll
-        for (int i = 0; i < DIM; ++i) L.ghat[(uint64_t)i * L.total_items + s.item] = (double)gv[i] * e0;
+            for (int i = 0; i < DIM; ++i) L.ghat[(uint64_t)i * L.total_items + item] = (double)gv[i] * e0;
+          }
+        }
       }
     }
     if (!WW) st_steps += s.k;
@@ -348,12 +375,13 @@ __global__ void __launch_bounds__(kWalkBlock,
     active = false;
   };
   // Plain, drift and batched walks: a lane whose walk ended waits (with its closest point,
-  // gamma and capped flag) until kDeferLanes lanes of the warp have ended, or the work is
+  // gamma and capped flag) until kGather lanes of the warp have ended, or the work is
   // exhausted; they then add g, finish their walks and claim new ones together.  The two
   // divergent blocks (end and regeneration, run by one or two lanes) then run about once per
-  // kDeferLanes walk ends instead of in most iterations, while the waiting lanes sit out a
+  // kGather walk ends instead of in most iterations, while the waiting lanes sit out a
   // few steps.
   constexpr bool DEFER = !WW && !MESH;
+  constexpr int kGather = (GRAD && WOS_WALK_DEFER_LANES < 8) ? 8 : WOS_WALK_DEFER_LANES;
 #if defined(WOS_JIT_FIELDS)
   constexpr int kForm = GRAD ? 2 : 0;  // see green_q3
 #else
@@ -365,7 +393,7 @@ __global__ void __launch_bounds__(kWalkBlock,
   for (;;) {
     // ---- regeneration: lanes without a walk claim the next items ----
     unsigned need = __ballot_sync(kFull, !active);
-    if (!DEFER || exhausted || __popc(need) >= kDeferLanes) {
+    if (!DEFER || exhausted || __popc(need) >= kGather) {
       if (DEFER && pend) {
         const DevProblem<R>& Pe = BATCHED ? Pall[s.prob] : *Pshared;
         if (!pcap) s.acc += s.W * w_exp(pgam) * g_at<DIM>(Pe, pxb);   // Alg. 1: g at the closest point
@@ -403,7 +431,7 @@ __global__ void __launch_bounds__(kWalkBlock,
       }
     }
     if (__ballot_sync(kFull, active) == 0u) break;
-    if (MESH) {
+    if constexpr (MESH) {
       // Distance queries.  A query visits anything from a handful of nodes near the boundary to
       // hundreds deep inside, so lanes that all wait for the warp's longest one idle most of the
       // time (5.3 of 32 lanes active with certified radii, 3.1 with exact ones).  Each lane keeps
@@ -696,7 +724,7 @@ __global__ void __launch_bounds__(kWalkBlock,
 
   if (accumulate && acc_p != kNoPoint) {
     double e0 = point_factor<DIM, R>(L, BATCHED ? Pall[acc_prob] : *Pshared, acc_p);
-    if (!GRAD) {
+    if (!SUM64) {
       double c = (double)sh, n = (double)n_acc;
       s1 = n * c + (double)d1;
       s2 = n * c * c + 2.0 * c * (double)d1 + (double)d2;
@@ -778,9 +806,11 @@ cudaError_t launch_walks_t(const WalkLaunch& L, int num_sms, cudaStream_t stream
     return (DIM == 3 && L.mesh) ? launch_walks_m<DIM, R, true, false, false, true>(L, num_sms, stream)
                                 : launch_walks_m<DIM, R, false, false, false, true>(L, num_sms, stream);
   const bool ww = L.ww_lo > 0.0;
-  if (sizeof(R) == 4 && !ww && !L.mesh && L.regs_variant != 0)
-    return (L.regs_variant == 1) ? launch_walks_m<DIM, R, false, false, false, false, false, 8>(L, num_sms, stream)
-                                 : launch_walks_m<DIM, R, false, false, false, false, false, 4>(L, num_sms, stream);
+  if constexpr (sizeof(R) == 4) {
+    if (!ww && !L.mesh && L.regs_variant != 0)
+      return (L.regs_variant == 1) ? launch_walks_m<DIM, R, false, false, false, false, false, 8>(L, num_sms, stream)
+                                   : launch_walks_m<DIM, R, false, false, false, false, false, 4>(L, num_sms, stream);
+  }
   if (DIM == 3 && L.mesh)
     return ww ? launch_walks_m<DIM, R, true, false, true>(L, num_sms, stream)
               : launch_walks_m<DIM, R, true, false, false>(L, num_sms, stream);
