@@ -30,8 +30,8 @@ struct wos_ctx {
   float* radial_tab[2] = {nullptr, nullptr};
   // buffers of wos_solve_host
   float* h_pts = nullptr;
-  double* h_acc = nullptr;  // sum, sumsq, mean, var, se: 5 * cap doubles
-  int64_t* h_count = nullptr;
+  double* h_acc = nullptr;  // sum, sumsq, count, mean, var, se: 6 * cap words
+  double* h_out = nullptr;  // page-locked: mean, var, se and the statistics (small calls)
   int64_t host_cap = 0;
   // FP64 accumulators of wos_solve_mean / wos_solve_batched (sum, sumsq, count per point)
   double* mv_sum = nullptr;   // 2 * mv_cap doubles: sum, then sumsq
