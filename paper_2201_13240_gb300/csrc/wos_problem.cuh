@@ -79,7 +79,7 @@ struct DevProblem {
   const float* mesh_tris;   // 12 floats per triangle in leaf order, device
   int32_t ncsg;
   int32_t mg_res;           // mesh distance grid: nodes per axis (0: none)
-  int32_t mesh_top;         // the first mesh_top nodes are the tree's top levels (staged in shared memory)
+  int32_t mesh_top;         // the first mesh_top nodes are the tree's top levels (next-flight kernels stage them)
   int32_t pad3;
   const R* mgrid;           // exact distances at the grid nodes, x fastest, device
   const void* mg_pad_ptr;   // keeps the 16-byte layout
@@ -416,7 +416,7 @@ WOS_HD R g_at(const DevProblem<R>& P, const R* x) {
 // triangle so far.
 // ---------------------------------------------------------------------------
 constexpr int kMeshStack = 32;  // entries of the traversal stack (a full stack repeats the pass: mesh_query)
-constexpr int kMeshTopMax = 21;  // nodes of the BVH's top levels staged in shared memory (1 + 4 + 16)
+constexpr int kMeshTopMax = 21;  // nodes of the BVH's top levels, staged in shared memory by next-flight kernels (1 + 4 + 16)
 
 struct F4 {
   float x, y, z, w;
