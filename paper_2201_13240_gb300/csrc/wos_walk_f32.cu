@@ -62,38 +62,42 @@ __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__
   const uint32_t lane = threadIdx.x & 31, base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kChunkMin;
   if (base >= total) return;
   const uint32_t n = min((uint32_t)kChunkMin, total - base);
-  constexpr int Q = (int)kChunkMin / 32;
-  float a[Q];
-  uint32_t it[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const bool in = 32 * q + lane < n;
-    a[q] = in ? acc[base + 32 * q + lane] : 0.0f;
-    it[q] = in ? iters[base + 32 * q + lane] : 0u;
+  // The warp's walks, staged: a claim takes consecutive ones, so its loads have no bank conflicts (from
+  // registers by eight shuffles and selects, with the point a global load in every round, 2^20 walks took
+  // 28 us, so 22).
+  __shared__ float walk_acc[4][kChunkMin];
+  __shared__ uint32_t walk_iters[4][kChunkMin], walk_point[4][kChunkMin];
+  const uint32_t warp = threadIdx.x >> 5;
+  for (uint32_t i = lane; i < n; i += 32) {
+    walk_acc[warp][i] = acc[base + i];
+    walk_iters[warp][i] = iters[base + i];
+    walk_point[warp][i] = point[base + i];
   }
+  __syncwarp();
   // A lane's sums over consecutive walks of one point are a run; runs wait in shared memory until the
   // walks are through, so that their FP64 arithmetic is done by all lanes at once, and runs of one
   // point meet in one atomic (flushed as they end, by a lane or two: 2.6e5 points x 4 walks of the 3D
   // cube 808 us, so 680; 30 points x 8192 walks 386 us, so 299).
   __shared__ SumRun runs[4][kChunkMin];
-  SumRun* run = runs[threadIdx.x >> 5];
+  SumRun* run = runs[warp];
   uint32_t n_runs = 0;  // of the warp
   SumRun r = {0xffffffffu, 0u, 0.0f, 0.0f, 0.0f};
-  auto add = [&](bool on, uint32_t item, float v) {
-    const uint32_t q = on ? point[item] : r.p;
+  auto add = [&](bool on, uint32_t i) {
+    const uint32_t q = on ? walk_point[warp][i] : r.p;
     const bool ends = on && r.n != 0u && q != r.p;
     const unsigned done = __ballot_sync(kFull, ends);
     if (ends) run[n_runs + __popc(done & ((1u << lane) - 1u))] = r;
     n_runs += __popc(done);
     if (!on) return;
+    const float v = walk_acc[warp][i];
     if (q != r.p) r = SumRun{q, 0u, v, 0.0f, 0.0f};
     const float dv = v - r.sh;
     r.d1 += dv;
     r.d2 += dv * dv;
     ++r.n;
   };
-  add(lane < n, base + lane, a[0]);
-  uint32_t free_at = it[0];  // iteration at which the lane has no walk
+  add(lane < n, lane);
+  uint32_t free_at = (lane < n) ? walk_iters[warp][lane] : 0u;  // iteration at which the lane has no walk
   for (uint32_t next = 32; next < n;) {
     // the iteration of the next claim
     uint32_t t = __reduce_min_sync(kFull, free_at);
@@ -107,20 +111,9 @@ __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__
     }
     const unsigned claim = __ballot_sync(kFull, free_at <= t);
     const uint32_t j = next + __popc(claim & ((1u << lane) - 1u));
-    float v = 0.0f;
-    uint32_t k = 0;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const float vq = __shfl_sync(kFull, a[q], (int)(j & 31u));
-      const uint32_t kq = __shfl_sync(kFull, it[q], (int)(j & 31u));
-      if ((j >> 5) == (uint32_t)q) {
-        v = vq;
-        k = kq;
-      }
-    }
     const bool takes = (claim >> lane & 1u) && j < n;
-    add(takes, base + j, v);
-    if (takes) free_at = t + k;
+    add(takes, j);
+    if (takes) free_at = t + walk_iters[warp][j];
     next += __popc(claim);
   }
   const unsigned last = __ballot_sync(kFull, r.n != 0u);
