@@ -24,10 +24,10 @@ HOSTCHECK = os.path.join(HERE, "libwos_hostcheck.so")
 CU_SOURCES = ["wos_capi.cu", "wos_walk_f32.cu", "wos_walk_f64.cu", "wos_nf_f32.cu", "wos_nf_f64.cu",
               "wos_adjoint.cu", "wos_render.cu", "wos_jit.cu", "wos_mesh.cpp", "wos_handles.cu", "wos_peaks.cu"]
 HEADERS = ["wos_math.cuh", "wos_problem.cuh", "wos_walk_impl.cuh", "wos_nf_impl.cuh", "wos_adjoint_impl.cuh",
-           "wos_internal.h", "wos_mesh.h", "wos_jit.h", "wos_capi_state.h"]
+           "wos_internal.h", "wos_rules.h", "wos_mesh.h", "wos_jit.h", "wos_capi_state.h"]
 # headers of the walk kernel, embedded in the library for the runtime-compiled (problem-
 # specialised) kernels
-JIT_HEADERS = ["wos_internal.h", "wos_math.cuh", "wos_problem.cuh", "wos_walk_impl.cuh", "wos_adjoint_impl.cuh"]
+JIT_HEADERS = ["wos_internal.h", "wos_rules.h", "wos_math.cuh", "wos_problem.cuh", "wos_walk_impl.cuh", "wos_adjoint_impl.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC, "-I", BUILD_DIR]
 
@@ -105,7 +105,7 @@ def build_lib(force: bool = False, verbose: bool = False) -> str:
 
 def build_hostcheck(force: bool = False) -> str:
     src = os.path.join(CSRC, "wos_hostcheck.cpp")
-    deps = [src, os.path.join(CSRC, "wos_math.cuh")]
+    deps = [src, os.path.join(CSRC, "wos_math.cuh"), os.path.join(CSRC, "wos_rules.h")]
     if not force and not _stale(HOSTCHECK, deps):
         return HOSTCHECK
     tmp = HOSTCHECK + f".tmp{os.getpid()}"

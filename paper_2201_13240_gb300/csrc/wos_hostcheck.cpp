@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "wos_math.cuh"
+#include "wos_rules.h"
 
 extern "C" {
 
@@ -282,6 +283,10 @@ void wos_hc_mix_radius(int dim, int fp64, double a, double lam, const double* u,
     }
   }
 }
+
+// dispatch rules
+int wos_hc_sums_in_fp64(int grad, int gathers, int lanes) { return wos::sums_in_fp64(grad != 0, gathers != 0, lanes); }
+int wos_hc_finds_item_again(int gathers, int lanes) { return wos::finds_item_again(gathers != 0, lanes); }
 
 // FP32 uniforms of the walk kernels from Philox words
 void wos_hc_uniform_f32(const uint32_t* x, int64_t n, double* out) {

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #endif
+#include "wos_rules.h"
 
 namespace wos {
 

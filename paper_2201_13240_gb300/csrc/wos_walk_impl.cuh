@@ -247,11 +247,8 @@ __global__ void __launch_bounds__(kWalkBlock,
   double s1 = 0.0, s2 = 0.0;
   uint32_t n_acc = 0;
   R sh = R(0), d1 = R(0), d2 = R(0);  // FP32 partial sums shifted by the point's first value
-  // SUM64: s1 and s2 are the sums themselves.  Where six or eight ends are finished at a time two FP64
-  // additions a walk cost less than the shift (a batch 46.2 -> 45.3 ms, the 2D square 4.48 -> 4.37; at four
-  // the 3D cube 109.8 -> 110.2 ms), and the shifted FP32 sums lose digits when a
-  // point's first walk is an outlier of a heavy-tailed estimate.
-  constexpr bool SUM64 = GRAD || WOS_WALK_DEFER_LANES >= 6;
+  constexpr bool DEFER = !WW && !MESH;  // ended walks are gathered (below)
+  constexpr bool SUM64 = sums_in_fp64(GRAD, DEFER, WOS_WALK_DEFER_LANES);  // s1 and s2 are the sums themselves
   // spatial gradient: per-lane partial sums of (grad U - U grad gamma) and grad gamma(x_0)
   double gs1[3] = {0.0, 0.0, 0.0}, gs2[3] = {0.0, 0.0, 0.0};
   R ggam[3] = {R(0), R(0), R(0)};
@@ -274,10 +271,9 @@ __global__ void __launch_bounds__(kWalkBlock,
   const int ww_depth = WW ? (L.ww_depth < kWWDepth ? L.ww_depth : kWWDepth) : 0;
   const R ww_lo = R(L.ww_lo), ww_hi = R(L.ww_hi);
 
-  // the item of the lane's walk, for the per-walk outputs: carried (two registers), or found again from
-  // its point and walk id where the fields need the registers
+  // the item of the lane's walk, for the per-walk outputs
   auto item_of = [&]() -> uint64_t {
-    if (WOS_WALK_DEFER_LANES < 8) return s.item;
+    if (!finds_item_again(DEFER, WOS_WALK_DEFER_LANES)) return s.item;
     const uint64_t j = (uint64_t)(uint32_t)(s.w - (uint32_t)L.walk_offset);
     if (L.walk_end == nullptr) return (uint64_t)s.p * (uint64_t)L.walks_uniform + j;
     return (s.p > 0u ? (uint64_t)__ldg(&L.walk_end[s.p - 1u]) : 0ull) + j;
@@ -380,7 +376,6 @@ __global__ void __launch_bounds__(kWalkBlock,
   // divergent blocks (end and regeneration, run by one or two lanes) then run about once per
   // kGather walk ends instead of in most iterations, while the waiting lanes sit out a
   // few steps.
-  constexpr bool DEFER = !WW && !MESH;
   constexpr int kGather = (GRAD && WOS_WALK_DEFER_LANES < 8) ? 8 : WOS_WALK_DEFER_LANES;
 #if defined(WOS_JIT_FIELDS)
   constexpr int kForm = GRAD ? 2 : 0;  // see green_q3
