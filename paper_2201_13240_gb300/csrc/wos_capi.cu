@@ -409,17 +409,27 @@ int no_window(wos_ctx* ctx, const wos_params* prm) {
   return WOS_OK;
 }
 
-// The register cap of the generic FP32 value kernel (five blocks per SM otherwise).  3D B-spline
-// fields keep 64 taps' weights and indices: four blocks (a noise cube, 4096 points x 256 walks: 4 / 5 /
-// 6 / 8 blocks 4.21 / 4.70 / 5.38 / 5.94 ms; in 2D 4.77 / 4.51 / 4.46 / 4.81).  Closed-form fields keep
-// little and wait on the interpreter's chains: eight, where there are walks enough to fill them
-// (2D square 8.4e6 walks 6.24 / 5.58 / 5.27 / 5.07 ms, 3D cube 4.2e6 walks 8.77 / 7.91 / 7.46 / 7.21; a
-// solve of 2.6e5 walks 441 / 437 / 450 / 495 us).
-int generic_variant(const DevProblem<double>& P, uint64_t total) {
+bool has_bspline(const DevProblem<double>& P) {
   const wos::DevField<double>* fields[6] = {&P.alpha, &P.phi, &P.sigma, &P.f, &P.g, &P.um};
   for (const wos::DevField<double>* f : fields)
-    if (f->kind == wos::F_GRID_BSPLINE) return P.dim == 3 ? 2 : 0;
-  return total > wos::kSpreadItems ? 1 : 0;
+    if (f->kind == wos::F_GRID_BSPLINE) return true;
+  return false;
+}
+
+// The generic FP32 walk kernel's launches for a solve: small solves (per-walk buffers in L) spread their
+// walks over the whole chip, and walk_sum_kernel adds them up (launch_walk_sums, by the caller).  With
+// per-point counts the number of walks is on the device only: both forms are launched, and one of them
+// returns at once.  bspline: of a problem's fields; batches choose their register cap by a schedule.
+cudaError_t launch_generic_f32(wos::WalkLaunch L, int num_sms, bool bspline, cudaStream_t st) {
+  const bool batch = L.probs != nullptr;
+  if (L.item_acc != nullptr) {
+    if (!batch) L.regs_variant = wos::value_variant(L.dim, bspline, wos::walks_of_launch(L.total_items, true));
+    const cudaError_t e = (batch || L.walk_end != nullptr) ? wos::launch_walks_counts_f32(L, num_sms, st)
+                                                           : wos::launch_walks_small_f32(L, num_sms, st);
+    if (e != cudaSuccess || L.walk_end == nullptr) return e;
+  }
+  if (!batch) L.regs_variant = wos::value_variant(L.dim, bspline, wos::walks_of_launch(L.total_items, false));
+  return wos::launch_walks_f32(L, num_sms, st);
 }
 
 int launch(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts, const int64_t* walk_end,
@@ -471,7 +481,7 @@ int launch(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts
     return fail(ctx, WOS_EUNSUPPORTED, "an extra drift (omega) works with the plain solve only");
   const bool fp64 = prm->precision == WOS_FP64;
   // small FP32 solves spread their walks over the whole chip (walk_sum_kernel adds them up)
-  // (per-point walk counts: the total is on the device, and both kernels look at it there)
+  // (per-point walk counts: the total is on the device, and the kernels look at it there)
   const bool spread = !fp64 && !nf && !gsum && sum != nullptr && uhat == nullptr &&
                       npts <= (int64_t)wos::kSpreadItems && (walk_end != nullptr || total <= wos::kSpreadItems);
   if (spread) wos::use_spread(&L, ctx->spread);
@@ -489,8 +499,8 @@ int launch(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts
   } else {
     L.problem = prob->d32;
     L.problem_bytes = (int)sizeof(DevProblem<float>);
-    L.regs_variant = generic_variant(prob->host64, walk_end ? ~0ull : total);
-    e = nf ? wos::launch_nf_f32(L, ctx->num_sms, st) : wos::launch_walks_f32(L, ctx->num_sms, st);
+    e = nf ? wos::launch_nf_f32(L, ctx->num_sms, st)
+           : launch_generic_f32(L, ctx->num_sms, has_bspline(prob->host64), st);
   }
   if (e == cudaSuccess && spread) e = wos::launch_walk_sums(L, L.ww_lo == 0.0 && !L.mesh, st);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "walk kernel launch");
@@ -1654,7 +1664,7 @@ int solve_batch_impl(wos_ctx* ctx, const wos_batch* b, const wos_schedule& sched
   if (spread) wos::use_spread(&L, ctx->spread);
   cudaKernel_t spec = b->jit.kernel[fp64 ? 1 : 0][sched.regs_variant == 1 ? 1 : 0];
   if (spec != nullptr) e = wos::launch_walks_kernel(L, spec, fp64 ? 8 : 4, ctx->num_sms, st);  // wos_batch_specialize
-  else e = fp64 ? wos::launch_walks_f64(L, ctx->num_sms, st) : wos::launch_walks_f32(L, ctx->num_sms, st);
+  else e = fp64 ? wos::launch_walks_f64(L, ctx->num_sms, st) : launch_generic_f32(L, ctx->num_sms, false, st);
   if (e == cudaSuccess && spread) e = wos::launch_walk_sums(L, true, st);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "batched walk kernel launch");
   return WOS_OK;

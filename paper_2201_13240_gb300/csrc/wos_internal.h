@@ -18,11 +18,6 @@ enum {
   ST_MESH_NODES = 6, ST_MESH_TRIS = 7, ST_EXHAUSTED = 8, ST_WORDS = 9
 };
 
-// Largest launch (walks) that takes the per-walk buffers of a small solve (16 MB per context): about
-// ten walks for each lane of the chip; a larger launch keeps every lane busy by itself (1.67e6
-// walks: 1.02 ms either way).
-constexpr uint64_t kSpreadItems = 1ull << 20;
-
 struct WalkLaunch {
   const void* problem;            // DevProblem<R> in device memory
   int problem_bytes;              // sizeof(DevProblem<R>), multiple of 16
@@ -133,6 +128,9 @@ cudaError_t launch_adjoint_kernel(const AdjLaunch& L, cudaKernel_t kernel, int r
 
 // launch the persistent walk kernel; returns a cudaError_t
 cudaError_t launch_walks_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream);
+// small solves' forms (SpreadForm): equal counts; per-point counts and batches
+cudaError_t launch_walks_small_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream);
+cudaError_t launch_walks_counts_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream);
 cudaError_t launch_walks_f64(const WalkLaunch& L, int num_sms, cudaStream_t stream);
 
 // a walk kernel compiled at run time for one problem (same parameter block and launch

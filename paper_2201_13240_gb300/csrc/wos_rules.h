@@ -2,6 +2,12 @@
 // CUDA so that the host check library can be asked for them too.
 #pragma once
 
+#if defined(__CUDACC_RTC__)
+#include "wos_math.cuh"  // fixed-width integer types of runtime compilation
+#else
+#include <stdint.h>
+#endif
+
 #if defined(__CUDACC__)
 #define WOS_RULE __host__ __device__ constexpr
 #else
@@ -22,5 +28,36 @@ WOS_RULE bool sums_in_fp64(bool grad, bool gathers, int lanes) { return grad || 
 // point and walk id where eight lanes are gathered, that is where the fields need the registers (B-spline
 // fields 7.57 -> 7.43 ms; the 3D cube 109.7 -> 111.2).
 WOS_RULE bool finds_item_again(bool gathers, int lanes) { return gathers && lanes >= 8; }
+
+// Largest launch (walks) that takes the per-walk buffers of a small solve (16 MB per context): about
+// ten walks for each lane of the chip; a larger launch keeps every lane busy by itself (1.67e6
+// walks: 1.02 ms either way).
+constexpr uint64_t kSpreadItems = 1ull << 20;
+
+// Form of a walk kernel: its walks' sums are formed in the kernel, left to walk_sum_kernel, or either, by the
+// number of walks in the launch.  As a choice at a walk's end it costs large solves up to 5 % (2D B-spline
+// annulus, 4.2e6 walks, 4.30 -> 4.51 ms; noise cube at five blocks 8.94 -> 9.05 ms), so of the generic kernels
+// large solves run the first form (4.35 ms).  Small solves with per-point counts, and small batches, run the
+// second: 3 to 11 % faster than the third.  Small solves of equal counts keep the third: they wait for a lone
+// walk's steps, and those are the faster in it (4096 x 256 windows 18.8 ms against 21.3, the 2D square's 32^2 x
+// 256 walks 475 us against 530; 20.6 ms and 522 us in one module with the batches' kernels).  Compiled kernels hold the choice: a second kernel would add half to their compilation (0.1 to
+// 0.8 s), and it costs nothing but in 3D windows (1.20 -> 1.22 ms).
+enum SpreadForm { SPREAD_NEVER = 0, SPREAD_ALWAYS = 1, SPREAD_BY_SIZE = 2 };
+
+// The register cap of the generic FP32 value kernel for a launch of `walks` walks: variant 0, five blocks
+// per SM; 1, eight; 2, four.  3D B-spline fields keep 64 taps' weights and indices: four blocks (a noise cube,
+// 4096 points x 256 walks: 4 / 5 / 6 / 8 blocks 4.21 / 4.70 / 5.38 / 5.94 ms; in 2D 4.77 / 4.51 / 4.46 /
+// 4.81).  Closed-form fields keep little and wait on the interpreter's chains: eight, where there are
+// walks enough to fill them (2D square 8.4e6 walks 6.24 / 5.58 / 5.27 / 5.07 ms, 3D cube 4.2e6 walks 8.77 /
+// 7.91 / 7.46 / 7.21; a solve of 2.6e5 walks 441 / 437 / 450 / 495 us).
+WOS_RULE int value_variant(int dim, bool bspline, uint64_t walks) {
+  return bspline ? (dim == 3 ? 2 : 0) : (walks > kSpreadItems ? 1 : 0);
+}
+
+// The most walks of a launch whose total is `total`, or known on the device only (per-point counts: ~0).  Of
+// those, the small solves' launch serves at most kSpreadItems walks and the other one more.
+WOS_RULE uint64_t walks_of_launch(uint64_t total, bool small_launch) {
+  return small_launch && total > kSpreadItems ? kSpreadItems : total;
+}
 
 }  // namespace wos

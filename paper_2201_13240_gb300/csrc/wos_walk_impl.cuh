@@ -191,12 +191,18 @@ constexpr int kMeshLeaves = 5;
 #define WOS_WALK_KERNEL wos_walk_kernel
 #endif
 // MINB > 0 overrides the resident-block target (the batched launches' high-occupancy variant, chosen by
-// the schedule, and the value kernel's variants by fields and size, see generic_variant).
-template <int DIM, typename R, bool MESH, bool BATCHED, bool WW, bool GRAD, bool DRIFT = false, int MINB = 0>
+// the schedule, and the value kernel's variants by fields and size, see value_variant).
+// SPREAD: see SpreadForm.
+template <int DIM, typename R, bool MESH, bool BATCHED, bool WW, bool GRAD, bool DRIFT = false, int MINB = 0,
+          int SPREAD = SPREAD_BY_SIZE>
 __global__ void __launch_bounds__(kWalkBlock,
                                   (sizeof(R) == 4) ? (GRAD ? 5 : (MESH ? kMeshBlocks : (MINB > 0 ? MINB : WOS_WALK_MIN_BLOCKS))) : 1)
     WOS_WALK_KERNEL(WalkLaunch L) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  // with per-point walk counts the total is the last inclusive prefix sum
+  const uint64_t total = (L.walk_end != nullptr) ? (uint64_t)__ldg(&L.walk_end[L.npts - 1]) : L.total_items;
+  // the form for another size (per-point counts launch both)
+  if (SPREAD != SPREAD_BY_SIZE && L.item_acc != nullptr && (total <= kSpreadItems) != (SPREAD == SPREAD_ALWAYS)) return;
   // stage the problem description (a few KB, read by every lane every step) in shared memory
   if (!BATCHED) {
     const int4* src = reinterpret_cast<const int4*>(L.problem);
@@ -223,15 +229,14 @@ __global__ void __launch_bounds__(kWalkBlock,
   const R s_root0 = w_sqrt(R(L.sigma_bar)), inv_sb0 = R(1) / R(L.sigma_bar);
   const uint32_t max_k = (L.max_steps >= (int64_t)0xffffffffll) ? 0xffffffffu : (uint32_t)L.max_steps;
 
-  // with per-point walk counts the total is the last inclusive prefix sum
-  const uint64_t total = (L.walk_end != nullptr) ? (uint64_t)__ldg(&L.walk_end[L.npts - 1]) : L.total_items;
   const bool accumulate = (L.sum != nullptr);
   uint64_t chunk = total / ((uint64_t)gridDim.x * (kWalkBlock / 32) * kChunksPerWarp);
   chunk = (chunk < kChunkMin) ? kChunkMin : (chunk > kChunkMax ? kChunkMax : chunk & ~31ull);
   if (L.chunk != 0u) chunk = L.chunk;  // a schedule's choice (a multiple of 32, checked by the host)
   // small solves: one walk per lane and claim, so that the walks of a launch that does not
   // fill the chip run side by side; their sums are left to walk_sum_kernel
-  const bool spread = sizeof(R) == 4 && !GRAD && L.item_acc != nullptr && total <= kSpreadItems;
+  const bool spread = SPREAD == SPREAD_ALWAYS || (SPREAD == SPREAD_BY_SIZE && sizeof(R) == 4 && !GRAD &&
+                                                  L.item_acc != nullptr && total <= kSpreadItems);
   if (spread || (GRAD && total <= kSpreadItems)) chunk = 32;
   uint64_t chunk_next = 0, chunk_end = 0;
   uint32_t cur_p = 0, cur_prob = 0;
@@ -765,18 +770,18 @@ __global__ void __launch_bounds__(kWalkBlock,
 
 #if !defined(__CUDACC_RTC__)
 template <int DIM, typename R, bool MESH, bool BATCHED, bool WW, bool GRAD = false, bool DRIFT = false,
-          int MINB = 0>
+          int MINB = 0, int SPREAD = SPREAD_NEVER>
 cudaError_t launch_walks_m(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
   size_t smem = BATCHED ? 0 : (size_t)L.problem_bytes;
   if (MESH) smem += (sizeof(int) + sizeof(R)) * kMeshStack * kWalkBlock + kWalkBlock;
   if (smem > 48 * 1024) {
-    cudaError_t ea = cudaFuncSetAttribute(wos_walk_kernel<DIM, R, MESH, BATCHED, WW, GRAD, DRIFT, MINB>,
+    cudaError_t ea = cudaFuncSetAttribute(wos_walk_kernel<DIM, R, MESH, BATCHED, WW, GRAD, DRIFT, MINB, SPREAD>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (ea != cudaSuccess) return ea;
   }
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &per_sm, wos_walk_kernel<DIM, R, MESH, BATCHED, WW, GRAD, DRIFT, MINB>, kWalkBlock, smem);
+      &per_sm, wos_walk_kernel<DIM, R, MESH, BATCHED, WW, GRAD, DRIFT, MINB, SPREAD>, kWalkBlock, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
   if (L.blocks_per_sm > 0 && L.blocks_per_sm < per_sm) per_sm = L.blocks_per_sm;
@@ -787,37 +792,46 @@ cudaError_t launch_walks_m(const WalkLaunch& L, int num_sms, cudaStream_t stream
   if ((uint64_t)grid > blocks_needed) grid = (int)(blocks_needed > 0 ? blocks_needed : 1);
   WalkLaunch arg = L;
   philox_round_keys(arg.seed, arg.rk);
-  wos_walk_kernel<DIM, R, MESH, BATCHED, WW, GRAD, DRIFT, MINB><<<grid, kWalkBlock, smem, stream>>>(arg);
+  wos_walk_kernel<DIM, R, MESH, BATCHED, WW, GRAD, DRIFT, MINB, SPREAD><<<grid, kWalkBlock, smem, stream>>>(arg);
   return cudaGetLastError();
 }
 
-template <int DIM, typename R>
+template <int DIM, typename R, int SPREAD = SPREAD_NEVER>
 cudaError_t launch_walks_t(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
-  if (L.probs != nullptr)
-    return (L.regs_variant == 1) ? launch_walks_m<DIM, R, false, true, false, false, false, 8>(L, num_sms, stream)
-                                 : launch_walks_m<DIM, R, false, true, false>(L, num_sms, stream);
-  if (L.drift) return launch_walks_m<DIM, R, false, false, false, false, true>(L, num_sms, stream);
-  if (L.gsum != nullptr || L.ghat != nullptr)  // spatial gradient (no weight window)
-    return (DIM == 3 && L.mesh) ? launch_walks_m<DIM, R, true, false, false, true>(L, num_sms, stream)
-                                : launch_walks_m<DIM, R, false, false, false, true>(L, num_sms, stream);
-  const bool ww = L.ww_lo > 0.0;
-  if constexpr (sizeof(R) == 4) {
-    if (!ww && !L.mesh && L.regs_variant != 0)
-      return (L.regs_variant == 1) ? launch_walks_m<DIM, R, false, false, false, false, false, 8>(L, num_sms, stream)
-                                   : launch_walks_m<DIM, R, false, false, false, false, false, 4>(L, num_sms, stream);
+  if constexpr (SPREAD != SPREAD_BY_SIZE)
+    if (L.probs != nullptr)
+      return (L.regs_variant == 1)
+                 ? launch_walks_m<DIM, R, false, true, false, false, false, 8, SPREAD>(L, num_sms, stream)
+                 : launch_walks_m<DIM, R, false, true, false, false, false, 0, SPREAD>(L, num_sms, stream);
+  if (L.drift) return launch_walks_m<DIM, R, false, false, false, false, true, 0, SPREAD>(L, num_sms, stream);
+  if constexpr (SPREAD == SPREAD_NEVER) {
+    if (L.gsum != nullptr || L.ghat != nullptr) {  // spatial gradient (no weight window)
+      if constexpr (DIM == 3)
+        if (L.mesh) return launch_walks_m<DIM, R, true, false, false, true>(L, num_sms, stream);
+      return launch_walks_m<DIM, R, false, false, false, true>(L, num_sms, stream);
+    }
   }
-  if (DIM == 3 && L.mesh)
-    return ww ? launch_walks_m<DIM, R, true, false, true>(L, num_sms, stream)
-              : launch_walks_m<DIM, R, true, false, false>(L, num_sms, stream);
-  return ww ? launch_walks_m<DIM, R, false, false, true>(L, num_sms, stream)
-            : launch_walks_m<DIM, R, false, false, false>(L, num_sms, stream);
+  const bool ww = L.ww_lo > 0.0;
+  if constexpr (DIM == 3)
+    if (L.mesh)
+      return ww ? launch_walks_m<DIM, R, true, false, true, false, false, 0, SPREAD>(L, num_sms, stream)
+                : launch_walks_m<DIM, R, true, false, false, false, false, 0, SPREAD>(L, num_sms, stream);
+  if (ww) return launch_walks_m<DIM, R, false, false, true, false, false, 0, SPREAD>(L, num_sms, stream);
+  if constexpr (sizeof(R) == 4) {  // value_variant
+    if constexpr (SPREAD == SPREAD_NEVER)
+      if (L.regs_variant == 1) return launch_walks_m<DIM, R, false, false, false, false, false, 8>(L, num_sms, stream);
+    if constexpr (DIM == 3)
+      if (L.regs_variant == 2)
+        return launch_walks_m<DIM, R, false, false, false, false, false, 4, SPREAD>(L, num_sms, stream);
+  }
+  return launch_walks_m<DIM, R, false, false, false, false, false, 0, SPREAD>(L, num_sms, stream);
 }
 
 template <int DIM, typename R>
 int blocks_per_sm_t() {
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wos_walk_kernel<DIM, R, false, false, false, false>, kWalkBlock,
-                                                sizeof(DevProblem<R>));
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wos_walk_kernel<DIM, R, false, false, false, false, false, 0, SPREAD_NEVER>,
+                                                kWalkBlock, sizeof(DevProblem<R>));
   return per_sm;
 }
 #endif  // !__CUDACC_RTC__

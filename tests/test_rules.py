@@ -20,3 +20,23 @@ def test_only_gathered_ends_change_the_sums(hc, lanes):
     assert bool(hc.wos_hc_sums_in_fp64(0, 1, lanes)) == (lanes >= 6)
     assert bool(hc.wos_hc_finds_item_again(1, lanes)) == (lanes == 8)
     assert hc.wos_hc_sums_in_fp64(1, 0, lanes) and hc.wos_hc_sums_in_fp64(1, 1, lanes)
+
+
+def test_register_variants_by_the_walks_of_a_launch(hc):
+    """Per-point counts are launched twice, at most 2^20 walks in the small form: that launch takes the
+    variant of small solves, whatever the total on the device, the other one that of large ones."""
+    for f in (hc.wos_hc_walks_of_launch,):
+        f.argtypes, f.restype = [C.c_uint64, C.c_int], C.c_uint64
+    hc.wos_hc_value_variant.argtypes = [C.c_int, C.c_int, C.c_uint64]
+    limit, unknown = 1 << 20, (1 << 64) - 1
+
+    def variant(dim, bspline, total, small):
+        return hc.wos_hc_value_variant(dim, bspline, hc.wos_hc_walks_of_launch(total, small))
+    for dim in (2, 3):
+        assert variant(dim, 0, unknown, 1) == 0 and variant(dim, 0, unknown, 0) == 1
+        for total in (1, limit):
+            assert variant(dim, 0, total, 1) == variant(dim, 0, total, 0) == 0
+        assert variant(dim, 0, limit + 1, 0) == 1
+        for total in (1, limit, limit + 1, unknown):
+            for small in (0, 1):
+                assert variant(dim, 1, total, small) == (2 if dim == 3 else 0)
