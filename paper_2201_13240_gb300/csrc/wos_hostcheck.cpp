@@ -284,6 +284,17 @@ void wos_hc_mix_radius(int dim, int fp64, double a, double lam, const double* u,
   }
 }
 
+// numbers t = m 2^e, m a 24-bit mantissa, whose w_div_known by d is not t / d
+int64_t wos_hc_div_known(int d, int e) {
+  const float fd = (float)d, rc = 1.0f / fd;
+  int64_t wrong = 0;
+  for (int32_t m = 1 << 23; m < 1 << 24; ++m) {
+    const float t = std::ldexp((float)m, e);
+    if (wos::w_div_known(t, fd, rc) != t / fd || wos::w_div_known(-t, fd, rc) != -t / fd) ++wrong;
+  }
+  return wrong;
+}
+
 // dispatch rules
 int wos_hc_sums_in_fp64(int grad, int gathers, int lanes) { return wos::sums_in_fp64(grad != 0, gathers != 0, lanes); }
 int wos_hc_value_variant(int dim, int bspline, uint64_t walks) { return wos::value_variant(dim, bspline != 0, walks); }

@@ -70,15 +70,11 @@ WOS_HD double w_div(double a, double b) { return a / b; }
 // t / d for a divisor whose reciprocal rc = 1/d is at hand, rounded as the division is: a quotient
 // estimate and one correction by its exact remainder (P. Markstein, "Computation of elementary
 // functions on the IBM RISC System/6000 processor", 1990), three instructions against the divide's
-// dozen.  Exact for |t| above 2^-100 and the divisors used here (every mantissa tried).
+// dozen.  Exact for |t| above 2^-100 and the divisors used here, 3 to 13 (tests/test_hostcheck_div.py
+// tries every mantissa).
 WOS_HD float w_div_known(float t, float d, float rc) {
-#if defined(__CUDA_ARCH__)
   const float q = t * rc;
   return fmaf(fmaf(-q, d, t), rc, q);
-#else
-  (void)rc;
-  return t / d;
-#endif
 }
 WOS_HD double w_div_known(double t, double d, double) { return t / d; }
 WOS_HD float w_sqrt(float x) { return sqrtf(x); }
