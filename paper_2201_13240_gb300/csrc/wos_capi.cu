@@ -432,6 +432,23 @@ cudaError_t launch_generic_f32(wos::WalkLaunch L, int num_sms, bool bspline, cud
   return wos::launch_walks_f32(L, num_sms, st);
 }
 
+// The FP32 next-flight kernel's launches for a solve: one, or where the number of walks is on the device
+// and decides, one for few walks and one for many.
+cudaError_t launch_nf_sized(wos::WalkLaunch L, int num_sms, bool bspline, cudaStream_t st) {
+  auto blocks = [&](uint64_t walks) { return wos::nf_blocks(L.dim, L.mesh != 0, L.nf_series > 0, bspline, walks); };
+  const uint64_t few = wos::nf_few_walks(bspline);
+  if (L.walk_end != nullptr && blocks(few) != blocks(L.total_items)) {
+    L.regs_variant = blocks(few);
+    L.nf_at_most = few;
+    const cudaError_t e = wos::launch_nf_f32(L, num_sms, st);
+    if (e != cudaSuccess) return e;
+    L.nf_at_most = 0;
+    L.nf_more_than = few;
+  }
+  L.regs_variant = blocks(L.total_items);
+  return wos::launch_nf_f32(L, num_sms, st);
+}
+
 int launch(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts, const int64_t* walk_end,
            int64_t walks_uniform, uint64_t total, const wos_params* prm, double* sum, double* sumsq,
            int64_t* count, uint64_t* stats, double* uhat, int64_t* steps, cudaStream_t st,
@@ -499,8 +516,8 @@ int launch(wos_ctx* ctx, const wos_problem* prob, const float* pts, int64_t npts
   } else {
     L.problem = prob->d32;
     L.problem_bytes = (int)sizeof(DevProblem<float>);
-    e = nf ? wos::launch_nf_f32(L, ctx->num_sms, st)
-           : launch_generic_f32(L, ctx->num_sms, has_bspline(prob->host64), st);
+    const bool bspline = has_bspline(prob->host64);
+    e = nf ? launch_nf_sized(L, ctx->num_sms, bspline, st) : launch_generic_f32(L, ctx->num_sms, bspline, st);
   }
   if (e == cudaSuccess && spread) e = wos::launch_walk_sums(L, L.ww_lo == 0.0 && !L.mesh, st);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "walk kernel launch");

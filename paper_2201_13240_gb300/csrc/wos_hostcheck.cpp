@@ -299,6 +299,9 @@ int64_t wos_hc_div_known(int d, int e) {
 int wos_hc_sums_in_fp64(int grad, int gathers, int lanes) { return wos::sums_in_fp64(grad != 0, gathers != 0, lanes); }
 int wos_hc_value_variant(int dim, int bspline, uint64_t walks) { return wos::value_variant(dim, bspline != 0, walks); }
 uint64_t wos_hc_walks_of_launch(uint64_t total, int small_launch) { return wos::walks_of_launch(total, small_launch != 0); }
+int wos_hc_nf_blocks(int dim, int mesh, int series, int bspline, uint64_t walks) {
+  return wos::nf_blocks(dim, mesh != 0, series != 0, bspline != 0, walks);
+}
 int wos_hc_finds_item_again(int gathers, int lanes) { return wos::finds_item_again(gathers != 0, lanes); }
 
 // FP32 uniforms of the walk kernels from Philox words

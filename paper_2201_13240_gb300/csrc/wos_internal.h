@@ -60,7 +60,7 @@ struct WalkLaunch {
   int drift;                      // the problem has an extra drift (omega fields)
   // launch schedule (0 = the kernel's own rule): walks claimed per warp at a time, resident
   // blocks launched per SM, and the register-cap variant of batched and generic FP32 value launches
-  // (1: 8 blocks/SM, 2, not batched: 4)
+  // (1: 8 blocks/SM, 2, not batched: 4); next-flight launches: resident blocks per SM
   uint32_t chunk;
   int32_t blocks_per_sm;
   int32_t regs_variant;
@@ -74,6 +74,9 @@ struct WalkLaunch {
   // Philox round keys of `seed`, set by the launch functions (philox_round_keys): in the
   // kernel's parameter space each round's key is a constant operand of the XOR
   uint32_t rk[20];
+  // next-flight launches with the number of walks on the device: the kernel returns at once unless it
+  // is more than nf_more_than and at most nf_at_most (0: no limit)
+  uint64_t nf_more_than, nf_at_most;
 };
 
 enum { ADJ_SIGMA = 0, ADJ_ALPHA = 1 };

@@ -37,13 +37,16 @@ namespace wos {
 constexpr int kNfBlock = 128;
 constexpr uint64_t kNfChunk = 128;
 
-// Resident blocks per SM: series 4 / 5 / 6 measured 21.6 / 20.7 / 21.1 ms, printed approximations 12.4 /
-// 11.9 / 10.9 ms (32^3 points x 96 walks of the 3D workload).  The kernel is bound by its code's size (a
+// MINB: resident blocks per SM in FP32, see nf_blocks.  The kernel is bound by its code's size (a
 // third of its stalls waited for instructions) and by the sweeps' arithmetic: the sweep split at the
-// last term, its loops rolled, and divisions by known integers took the series from 28.2 to 20.7 ms.
-template <int DIM, typename R, bool MESH, bool SERIES>
-__global__ void __launch_bounds__(kNfBlock, (sizeof(R) == 4) ? (SERIES ? 5 : 6) : 1) wos_nf_kernel(WalkLaunch L) {
+// last term, its loops rolled, and divisions by known integers took the series from 28.2 to 20.7 ms
+// (32^3 points x 96 walks of the 3D workload, 8 terms).
+template <int DIM, typename R, bool MESH, bool SERIES, int MINB>
+__global__ void __launch_bounds__(kNfBlock, (sizeof(R) == 4) ? MINB : 1) wos_nf_kernel(WalkLaunch L) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  const uint64_t total = (L.walk_end != nullptr) ? (uint64_t)__ldg(&L.walk_end[L.npts - 1]) : L.total_items;
+  if (L.nf_at_most != 0u && total > L.nf_at_most) return;
+  if (L.nf_more_than != 0u && total <= L.nf_more_than) return;
   {
     const int4* src = reinterpret_cast<const int4*>(L.problem);
     int4* dst = reinterpret_cast<int4*>(smem_raw);
@@ -75,7 +78,6 @@ __global__ void __launch_bounds__(kNfBlock, (sizeof(R) == 4) ? (SERIES ? 5 : 6) 
   const R cvol = (DIM == 2) ? R(3.14159265358979323846) : R(4.18879020478639098462);   // |B| / R^dim
   const R carea = (DIM == 2) ? R(6.28318530717958647692) : R(12.5663706143591729539);  // |dB| / R^(dim-1)
 
-  const uint64_t total = (L.walk_end != nullptr) ? (uint64_t)__ldg(&L.walk_end[L.npts - 1]) : L.total_items;
   const bool accumulate = (L.sum != nullptr);
   uint64_t chunk_next = 0, chunk_end = 0;
   bool exhausted = false, active = false;
@@ -368,18 +370,18 @@ __global__ void __launch_bounds__(kNfBlock, (sizeof(R) == 4) ? (SERIES ? 5 : 6) 
   }
 }
 
-template <int DIM, typename R, bool MESH, bool SERIES>
+template <int DIM, typename R, bool MESH, bool SERIES, int MINB>
 cudaError_t launch_nf_m(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
   size_t smem = (size_t)L.problem_bytes;
   if (MESH) smem += (sizeof(int) + sizeof(R)) * kMeshStack * kNfBlock + 128 * kMeshTopMax;
   if (smem > 48 * 1024) {
-    cudaError_t ea = cudaFuncSetAttribute(wos_nf_kernel<DIM, R, MESH, SERIES>,
+    cudaError_t ea = cudaFuncSetAttribute(wos_nf_kernel<DIM, R, MESH, SERIES, MINB>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (ea != cudaSuccess) return ea;
   }
   int per_sm = 0;
   cudaError_t e =
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wos_nf_kernel<DIM, R, MESH, SERIES>, kNfBlock, smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wos_nf_kernel<DIM, R, MESH, SERIES, MINB>, kNfBlock, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
   int grid = per_sm * num_sms;
@@ -389,18 +391,23 @@ cudaError_t launch_nf_m(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
   if ((uint64_t)grid > blocks_needed) grid = (int)(blocks_needed > 0 ? blocks_needed : 1);
   WalkLaunch arg = L;
   philox_round_keys(arg.seed, arg.rk);
-  wos_nf_kernel<DIM, R, MESH, SERIES><<<grid, kNfBlock, smem, stream>>>(arg);
+  wos_nf_kernel<DIM, R, MESH, SERIES, MINB><<<grid, kNfBlock, smem, stream>>>(arg);
   return cudaGetLastError();
 }
 
 template <int DIM, typename R>
 cudaError_t launch_nf_t(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
   const bool series = L.nf_series > 0;
-  if (DIM == 3 && L.mesh)
-    return series ? launch_nf_m<DIM, R, true, true>(L, num_sms, stream)
-                  : launch_nf_m<DIM, R, true, false>(L, num_sms, stream);
-  return series ? launch_nf_m<DIM, R, false, true>(L, num_sms, stream)
-                : launch_nf_m<DIM, R, false, false>(L, num_sms, stream);
+  if constexpr (DIM == 3)
+    if (L.mesh)
+      return series ? launch_nf_m<DIM, R, true, true, 4>(L, num_sms, stream)
+                    : launch_nf_m<DIM, R, true, false, 4>(L, num_sms, stream);
+  if constexpr (sizeof(R) == 4) {
+    if (series && L.regs_variant == 5) return launch_nf_m<DIM, R, false, true, 5>(L, num_sms, stream);
+    if (!series && L.regs_variant == 6) return launch_nf_m<DIM, R, false, false, 6>(L, num_sms, stream);
+  }
+  return series ? launch_nf_m<DIM, R, false, true, 4>(L, num_sms, stream)
+                : launch_nf_m<DIM, R, false, false, 4>(L, num_sms, stream);
 }
 
 }  // namespace wos

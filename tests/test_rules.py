@@ -40,3 +40,19 @@ def test_register_variants_by_the_walks_of_a_launch(hc):
         for total in (1, limit, limit + 1, unknown):
             for small in (0, 1):
                 assert variant(dim, 1, total, small) == (2 if dim == 3 else 0)
+
+
+def test_next_flight_register_caps(hc):
+    """More than four blocks per SM only where they are the faster ones: never on meshes or for few walks, and
+    never for the printed approximations with 3D B-spline fields, whose taps would spill."""
+    hc.wos_hc_nf_blocks.argtypes = [C.c_int] * 4 + [C.c_uint64]
+    for series in (0, 1):
+        for walks in (1, 1 << 18, 1 << 20, 1 << 30):
+            assert hc.wos_hc_nf_blocks(3, 1, series, 0, walks) == 4
+        for dim in (2, 3):
+            assert hc.wos_hc_nf_blocks(dim, 0, series, 0, 1 << 18) == 4
+            assert hc.wos_hc_nf_blocks(dim, 0, series, 1, 1 << 20) == 4
+            assert hc.wos_hc_nf_blocks(dim, 0, series, 0, (1 << 18) + 1) == (5 if series else 6)
+    assert hc.wos_hc_nf_blocks(3, 0, 0, 1, 1 << 30) == 4
+    assert hc.wos_hc_nf_blocks(2, 0, 0, 1, 1 << 30) == 6
+    assert hc.wos_hc_nf_blocks(3, 0, 1, 1, 1 << 30) == 5
