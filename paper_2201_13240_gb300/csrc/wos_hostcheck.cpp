@@ -302,6 +302,7 @@ uint64_t wos_hc_walks_of_launch(uint64_t total, int small_launch) { return wos::
 int wos_hc_nf_blocks(int dim, int mesh, int series, int bspline, uint64_t walks) {
   return wos::nf_blocks(dim, mesh != 0, series != 0, bspline != 0, walks);
 }
+int wos_hc_gradient_form(int compiled, int bspline) { return wos::gradient_form(compiled != 0, bspline != 0); }
 int wos_hc_finds_item_again(int gathers, int lanes) { return wos::finds_item_again(gathers != 0, lanes); }
 
 // FP32 uniforms of the walk kernels from Philox words

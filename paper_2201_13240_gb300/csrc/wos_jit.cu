@@ -258,7 +258,7 @@ std::string tuning(const DevProblem<double>& P, bool batch) {
   const int blocks = bspline ? (P.dim == 3 ? 4 : 5) : (P.dim == 3 ? (batch ? 7 : 6) : 8);
   const int gather = bspline ? 8 : (P.dim == 3 ? 4 : 6);
   return "#define WOS_WALK_MIN_BLOCKS " + std::to_string(blocks) + "\n#define WOS_WALK_DEFER_LANES " +
-         std::to_string(gather) + "\n";
+         std::to_string(gather) + "\n#define WOS_JIT_BSPLINE " + (bspline ? "1\n" : "0\n");
 }
 
 }  // namespace

@@ -464,8 +464,8 @@ struct FactPoly<R, OFF, K, NT, true> {
 // FORM (here and in Radial3) names the roundings of (1 - e^{-2a}) - 2a e^{-a}: 0 leaves the choice
 // to the compiler, 1 and 2 are w_one_minus_sq's with the rest fused.  They differ in the last bit,
 // but a walk's path depends on every bit; the gradient walks name the form that their kernels have
-// always had (generic 1, specialised 2), so that they stay the same walks however the kernel around
-// them is laid out.
+// always had (gradient_form), so that they stay the same walks however the kernel around them is
+// laid out.
 template <int FORM = 0>
 WOS_HD float green_q3(float a) {
   // q = (1 - a/sinh a)/a^2 = S(a) / (a^2 sinh a), S(a) = sinh a - a.  a < 1: S(a) = a^3 P(a^2)

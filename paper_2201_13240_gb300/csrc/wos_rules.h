@@ -34,6 +34,11 @@ WOS_RULE bool finds_item_again(bool gathers, int lanes) { return gathers && lane
 // walks: 1.02 ms either way).
 constexpr uint64_t kSpreadItems = 1ull << 20;
 
+// The rounding that a gradient walk's kernel names in the Green's-function norm (green_q3's FORM): the one
+// that kernels of its kind have always had, so that their walks stay the same.  Compiled kernels of
+// closed-form fields: 2; generic ones, and compiled ones with B-spline fields: 1.
+WOS_RULE int gradient_form(bool compiled, bool bspline) { return compiled && !bspline ? 2 : 1; }
+
 // Form of a walk kernel: its walks' sums are formed in the kernel, left to walk_sum_kernel, or either, by the
 // number of walks in the launch.  As a choice at a walk's end it costs large solves up to 5 % (2D B-spline
 // annulus, 4.2e6 walks, 4.30 -> 4.51 ms; noise cube at five blocks 8.94 -> 9.05 ms), so of the generic kernels

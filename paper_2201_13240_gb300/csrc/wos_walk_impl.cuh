@@ -382,10 +382,13 @@ __global__ void __launch_bounds__(kWalkBlock,
   // kGather walk ends instead of in most iterations, while the waiting lanes sit out a
   // few steps.
   constexpr int kGather = (GRAD && WOS_WALK_DEFER_LANES < 8) ? 8 : WOS_WALK_DEFER_LANES;
+#if !defined(WOS_JIT_BSPLINE)
+#define WOS_JIT_BSPLINE 0
+#endif
 #if defined(WOS_JIT_FIELDS)
-  constexpr int kForm = GRAD ? 2 : 0;  // see green_q3
+  constexpr int kForm = GRAD ? gradient_form(true, WOS_JIT_BSPLINE != 0) : 0;  // see green_q3
 #else
-  constexpr int kForm = GRAD ? 1 : 0;
+  constexpr int kForm = GRAD ? gradient_form(false, false) : 0;
 #endif
   bool pend = false, pcap = false;
   R pgam = R(0), pxb[3] = {R(0), R(0), R(0)};

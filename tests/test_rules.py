@@ -56,3 +56,10 @@ def test_next_flight_register_caps(hc):
     assert hc.wos_hc_nf_blocks(3, 0, 0, 1, 1 << 30) == 4
     assert hc.wos_hc_nf_blocks(2, 0, 0, 1, 1 << 30) == 6
     assert hc.wos_hc_nf_blocks(3, 0, 1, 1, 1 << 30) == 5
+
+
+def test_gradient_forms(hc):
+    """Compiled kernels of closed-form fields name their own rounding; generic kernels and those with B-spline
+    fields name the same one."""
+    assert hc.wos_hc_gradient_form(1, 0) == 2
+    assert hc.wos_hc_gradient_form(0, 0) == hc.wos_hc_gradient_form(0, 1) == hc.wos_hc_gradient_form(1, 1) == 1
