@@ -1015,10 +1015,6 @@ int wos_finalize(wos_ctx* ctx, const double* sum, const double* sumsq, const int
   return WOS_OK;
 }
 
-// results of up to this many points leave through a page-locked buffer (1.5 MB); larger ones spend
-// more on the second copy than on the waits
-static constexpr int64_t kHostStagePoints = 65536;
-
 int wos_solve_host(wos_ctx* ctx, const wos_problem* pr, const float* pts_host, int64_t npts, int32_t walks_uniform,
                    const wos_params* prm, double* mean_host, double* var_host, double* se_host,
                    uint64_t* stats_host, void* stream) {
@@ -1035,18 +1031,25 @@ int wos_solve_host(wos_ctx* ctx, const wos_problem* pr, const float* pts_host, i
     int64_t c1 = 0, c2 = 0;
     if (ctx->h_pts) cudaFree(ctx->h_pts);
     if (ctx->h_acc) cudaFree(ctx->h_acc);
-    if (ctx->h_out) cudaFreeHost(ctx->h_out);
     ctx->h_pts = nullptr;
     ctx->h_acc = nullptr;
-    ctx->h_out = nullptr;
     ctx->host_cap = 0;
     if ((rc = grow(ctx, &ctx->h_pts, 3 * npts, &c1, 1))) return rc;
     if ((rc = grow(ctx, &ctx->h_acc, 6 * npts, &c2, 1))) return rc;
-    if (npts <= kHostStagePoints && cudaMallocHost(&ctx->h_out, (3 * npts + wos::ST_WORDS) * sizeof(double)) != cudaSuccess) {
+    ctx->host_cap = npts;
+  }
+  // the page-locked buffer has its own capacity: a large call that does without leaves it be
+  const bool staged = wos::host_staged(npts);
+  if (staged && npts > ctx->out_cap) {
+    if (ctx->h_out) cudaFreeHost(ctx->h_out);
+    ctx->h_out = nullptr;
+    ctx->out_cap = 0;
+    if (cudaMallocHost(&ctx->h_out, (3 * npts + wos::ST_WORDS) * sizeof(double)) == cudaSuccess) {
+      ctx->out_cap = npts;
+    } else {
       cudaGetLastError();
       ctx->h_out = nullptr;  // the results are copied out one by one
     }
-    ctx->host_cap = npts;
   }
   // sum, sumsq and count (zeroed together), then mean, var and se (read back together)
   double* d_sum = ctx->h_acc;
@@ -1065,9 +1068,9 @@ int wos_solve_host(wos_ctx* ctx, const wos_problem* pr, const float* pts_host, i
   if (rc) return rc;
   rc = wos_finalize(ctx, d_sum, d_sumsq, d_count, npts, d_mean, d_var, d_se, stream);
   if (rc) return rc;
-  if (ctx->h_out != nullptr && npts <= kHostStagePoints) {
-    // Two copies into page-locked memory and one wait: a copy into a caller's pageable array waits for
-    // the stream by itself (5,003 points x 333 walks of the 3D cube: 1,013 us with four, so 990).
+  if (staged && ctx->h_out != nullptr) {
+    // two copies into page-locked memory and one wait (5,003 points x 333 walks of the 3D cube: 1,013 us with
+    // four copies that wait, so 990)
     e = cudaMemcpyAsync(ctx->h_out, d_mean, 3 * sizeof(double) * npts, cudaMemcpyDeviceToHost, st);
     double* st_out = ctx->h_out + 3 * npts;
     if (e == cudaSuccess)

@@ -31,8 +31,9 @@ struct wos_ctx {
   // buffers of wos_solve_host
   float* h_pts = nullptr;
   double* h_acc = nullptr;  // sum, sumsq, count, mean, var, se: 6 * cap words
-  double* h_out = nullptr;  // page-locked: mean, var, se and the statistics (small calls)
   int64_t host_cap = 0;
+  double* h_out = nullptr;  // page-locked: mean, var, se (out_cap points) and the statistics (host_staged)
+  int64_t out_cap = 0;
   // FP64 accumulators of wos_solve_mean / wos_solve_batched (sum, sumsq, count per point)
   double* mv_sum = nullptr;   // 2 * mv_cap doubles: sum, then sumsq
   int64_t* mv_count = nullptr;

@@ -80,4 +80,10 @@ WOS_RULE int nf_blocks(int dim, bool mesh, bool series, bool bspline, uint64_t w
   return bspline && dim == 3 ? 4 : 6;
 }
 
+// Whether wos_solve_host's results leave through a page-locked buffer, with one wait for the stream
+// (a copy into a caller's pageable array waits by itself).  Larger results spend more on the second copy
+// than on the waits: 8 walks per point of the 3D cube, copies per array / staged, us: 1,000 points 209 / 183,
+// 5,003 239 / 222, 10,000 270 / 263, 16,384 325 / 327, 30,000 380 / 403, 65,536 522 / 599.
+WOS_RULE bool host_staged(int64_t npts) { return npts <= 12288; }
+
 }  // namespace wos
