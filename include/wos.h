@@ -410,8 +410,9 @@ int wos_solve_batch(wos_ctx* ctx, const wos_batch* batch, const float* pts, cons
 /* Launch schedule of a batch's persistent launch (not in the paper).  The work queue
    hands each warp `chunk` consecutive (point, walk) items at a time: small chunks balance
    the tail, large ones keep a lane on one point (fewer partial-sum flushes).
-     chunk          0 = the kernel's rule (total / (warps x 64), 128..2048), else a
-                    multiple of 32 in 32..65536
+     chunk          0 = the kernel's rule (total / (warps x 64), 128..2048; FP32 launches of at
+                    most 2^20 walks with blocks_per_sm 0: one walk per lane, whose sums a second
+                    kernel forms), else a multiple of 32 in 32..65536
      blocks_per_sm  0 = as many 128-thread blocks as fit, else 1..32 (capped by what fits)
      regs_variant   0 = the default register cap, 1 = 64 registers (8 blocks per SM)
      reserved       0

@@ -1491,7 +1491,7 @@ extern "C" int wos_batch_specialized(const wos_batch* b, int32_t* flags_out, int
 namespace {
 int solve_batch_impl(wos_ctx* ctx, const wos_batch* b, const wos_schedule& sched, const float* pts,
                      const int32_t* walks, int32_t walks_uniform, const wos_params* prm, double* sum, double* sumsq,
-                     int64_t* count, uint64_t* stats, void* stream, bool trial = false);
+                     int64_t* count, uint64_t* stats, void* stream, bool large = false);
 
 bool valid_schedule(const wos_schedule& s) {
   const bool chunk_ok = s.chunk == 0 || (s.chunk >= 32 && s.chunk <= 65536 && s.chunk % 32 == 0);
@@ -1565,17 +1565,36 @@ extern "C" int wos_batch_autotune(wos_ctx* ctx, wos_batch* b, const float* pts, 
     cleanup();
     return cuda_fail(ctx, el, "autotune trial walks");
   }
+  // the walks of the launches that the schedule is for: above kSpreadItems they form their sums in the
+  // kernel, and so do the trials, however few walks they have
+  uint64_t solve_walks = (uint64_t)n * (uint64_t)std::max(walks_uniform, 0);
+  if (walks) {
+    int64_t last = 0;
+    walk_prefix_kernel<<<1, 1024, 0, st>>>(walks, n, b->walk_end);
+    cudaError_t ew = cudaGetLastError();
+    if (ew == cudaSuccess) ew = cudaMemcpyAsync(&last, b->walk_end + n - 1, sizeof(last), cudaMemcpyDeviceToHost, st);
+    if (ew == cudaSuccess) ew = cudaStreamSynchronize(st);
+    if (ew != cudaSuccess) {
+      cleanup();
+      return cuda_fail(ctx, ew, "autotune walk count");
+    }
+    solve_walks = (uint64_t)last;
+  }
+  const bool large = solve_walks > wos::kSpreadItems;
   // candidates: the kernel's own chunk rule and fixed chunks, at both register caps
   std::vector<wos_schedule> cand;
   const int32_t chunks[] = {0, 64, 128, 256, 512, 1024, 2048};
   for (int rv = 0; rv < 2; ++rv)
     for (int32_t c : chunks) cand.push_back(wos_schedule{c, 0, rv, 0});
-  double best = 1e300, dflt = -1.0;
-  wos_schedule best_s = cand[0];
+  // A small solve's trial takes a millisecond or two, and one of them says little: five rounds, each
+  // candidate's best.
+  const size_t rounds = large ? 1 : 5;
+  std::vector<double> took(cand.size(), 1e300);
   int rc = WOS_OK;
-  for (size_t i = 0; i <= cand.size() && rc == WOS_OK; ++i) {
+  for (size_t i = 0; i <= rounds * cand.size() && rc == WOS_OK; ++i) {
     // i == 0 warms up with the first candidate (untimed)
-    const wos_schedule& sc = cand[i == 0 ? 0 : i - 1];
+    const size_t at = i == 0 ? 0 : (i - 1) % cand.size();
+    const wos_schedule& sc = cand[at];
     cudaError_t em = cudaMemsetAsync(acc, 0, 2 * sizeof(double) * n, st);
     if (em == cudaSuccess) em = cudaMemsetAsync(cnt, 0, sizeof(int64_t) * n, st);
     if (em != cudaSuccess) {
@@ -1584,7 +1603,7 @@ extern "C" int wos_batch_autotune(wos_ctx* ctx, wos_batch* b, const float* pts, 
     }
     cudaEventRecord(e0, st);
     rc = solve_batch_impl(ctx, b, sc, pts, tw, 0, prm, acc, acc + n, cnt, reinterpret_cast<uint64_t*>(stt), stream,
-                          true);
+                          large);
     cudaEventRecord(e1, st);
     if (rc != WOS_OK) break;
     if (cudaEventSynchronize(e1) != cudaSuccess) {
@@ -1593,15 +1612,13 @@ extern "C" int wos_batch_autotune(wos_ctx* ctx, wos_batch* b, const float* pts, 
     }
     float ms = 0.0f;
     cudaEventElapsedTime(&ms, e0, e1);
-    if (i == 0) continue;
-    if (i == 1) dflt = ms;
-    if (ms < best) {
-      best = ms;
-      best_s = sc;
-    }
+    if (i > 0) took[at] = std::min(took[at], (double)ms);
   }
   cleanup();
   if (rc != WOS_OK) return rc;
+  const size_t fastest = (size_t)(std::min_element(took.begin(), took.end()) - took.begin());
+  const wos_schedule best_s = cand[fastest];
+  const double best = took[fastest], dflt = took[0];
   b->sched = best_s;
   if (best_out) *best_out = best_s;
   if (best_ms) *best_ms = best;
@@ -1620,7 +1637,7 @@ extern "C" int wos_solve_batch(wos_ctx* ctx, const wos_batch* b, const float* pt
 namespace {
 int solve_batch_impl(wos_ctx* ctx, const wos_batch* b, const wos_schedule& sched, const float* pts,
                      const int32_t* walks, int32_t walks_uniform, const wos_params* prm, double* sum, double* sumsq,
-                     int64_t* count, uint64_t* stats, void* stream, bool trial) {
+                     int64_t* count, uint64_t* stats, void* stream, bool large) {
   if (!b || b->ctx != ctx) return fail(ctx, WOS_EINVAL, "null batch or batch of another context");
   if (!prm) return fail(ctx, WOS_EINVAL, "params is NULL");
   if (!finite_pos(prm->eps) || prm->max_steps < 1 || (prm->precision != WOS_FP32 && prm->precision != WOS_FP64))
@@ -1677,9 +1694,9 @@ int solve_batch_impl(wos_ctx* ctx, const wos_batch* b, const wos_schedule& sched
   L.regs_variant = sched.regs_variant;
   const bool fp64 = prm->precision == WOS_FP64;
   L.probs = fp64 ? (const void*)b->d64 : (const void*)b->d32;
-  // small batches on the kernel's own schedule spread their walks (a set schedule, and the
-  // autotuner's trials, whose launches stand for larger ones, keep the persistent kernel's sums)
-  const bool spread = !fp64 && !trial && sched.chunk == 0 && sched.blocks_per_sm == 0 &&
+  // small batches on the kernel's own schedule spread their walks (a set schedule, and autotuner's
+  // trials that stand for a launch of more walks, `large`, keep the persistent kernel's sums)
+  const bool spread = !fp64 && !large && sched.chunk == 0 && sched.blocks_per_sm == 0 &&
                       b->npts <= (int64_t)wos::kSpreadItems && (walk_end != nullptr || total <= wos::kSpreadItems);
   if (spread) wos::use_spread(&L, ctx->spread);
   cudaKernel_t spec = b->jit.kernel[fp64 ? 1 : 0][sched.regs_variant == 1 ? 1 : 0];
