@@ -55,8 +55,7 @@ struct CsgF32 {
 };
 
 __device__ void csg_load_f32(const DevProblem<double>& P, CsgF32* C) {
-  const int n = P.domain_kind == D_CSG ? P.ncsg : 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = threadIdx.x; i < P.ncsg; i += blockDim.x) {
     C->node[i].prim = P.csg[i].prim;
     C->node[i].op = P.csg[i].op;
     float m = 0.0f;
@@ -116,9 +115,8 @@ __device__ int csg_decide(const CsgF32& C, int n, const float* xf, float X, floa
   return finite ? who : -1;
 }
 
-// sd_domain through csg_decide
+// sd_domain of a CSG list through csg_decide
 __device__ double sd_decided(const DevProblem<double>& P, const CsgF32& C, const double* x) {
-  if (P.domain_kind != D_CSG) return sd_domain(P, x);
   const float xf[3] = {(float)x[0], (float)x[1], (float)x[2]};
   float lo, hi;
   const int who = csg_decide(C, P.ncsg, xf, fabsf(xf[0]) + fabsf(xf[1]) + fabsf(xf[2]), &lo, &hi);
@@ -145,13 +143,17 @@ __device__ void put(uint8_t* rgba, int64_t i, const double* c) {
   rgba[4 * i + 3] = 255;
 }
 
+// CSG: the domain is a CSG list, and csg_decide chooses what a step evaluates.  A form of its own, since its
+// registers (86 a thread against 78) slowed the views of other domains down (a box 972 -> 1,018 us).
+template <bool CSG>
 __global__ void render3_kernel(const DevProblem<double>* Pg, View3 V, const double* sum, const int64_t* count,
                                uint8_t* rgba, float* value, float* depth) {
   const DevProblem<double>& P = *Pg;
   __shared__ CsgF32 C;
-  csg_load_f32(P, &C);
-  __syncthreads();
-  const bool csg = P.domain_kind == D_CSG;
+  if (CSG) {
+    csg_load_f32(P, &C);
+    __syncthreads();
+  }
   int64_t npx = (int64_t)V.width * V.height;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < npx; i += (int64_t)gridDim.x * blockDim.x) {
     int px = (int)(i % V.width), py = (int)(i / V.width);
@@ -169,7 +171,7 @@ __global__ void render3_kernel(const DevProblem<double>* Pg, View3 V, const doub
     // sphere-trace max(sdf_domain, sdf_keep): the domain behind the plane
     double t = 0.0, tmax = 1e3 * V.scale;
     float eyef[3], dirf[3], nf[3], orgf[3], eye1 = 0.0f, org1 = 0.0f;
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; CSG && k < 3; ++k) {
       eyef[k] = (float)V.eye[k];
       dirf[k] = (float)dir[k];
       nf[k] = (float)V.n[k];
@@ -184,7 +186,7 @@ __global__ void render3_kernel(const DevProblem<double>* Pg, View3 V, const doub
       // which of the domain's and the plane's distance is the larger, in FP32 where that suffices
       bool plane = true, domain = true;  // may be
       int who = -1;
-      if (csg) {
+      if (CSG) {
         const float tf = (float)t, X = eye1 + 1.75f * fabsf(tf);
         float xf[3], spf = 0.0f, lo, hi;
         for (int k = 0; k < 3; ++k) {
@@ -241,7 +243,7 @@ __global__ void render3_kernel(const DevProblem<double>* Pg, View3 V, const doub
             double xp[3] = {x[0], x[1], x[2]}, xm[3] = {x[0], x[1], x[2]};
             xp[k] += h;
             xm[k] -= h;
-            g[k] = sd_decided(P, C, xp) - sd_decided(P, C, xm);
+            g[k] = CSG ? sd_decided(P, C, xp) - sd_decided(P, C, xm) : sd_domain(P, xp) - sd_domain(P, xm);
           }
           double gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]) + 1e-300;
           double lam = 0.0;
@@ -370,7 +372,8 @@ int render_slice(const DevProblem<double>* dprob, const DevProblem<double>& host
     double span2 = 0.0;
     for (int k = 0; k < 3; ++k) span2 += (host.dom[3 + k] - host.dom[k]) * (host.dom[3 + k] - host.dom[k]);
     V.scale = sqrt(span2) > 0.0 ? sqrt(span2) : 1.0;
-    render3_kernel<<<blocks, 256, 0, st>>>(dprob, V, sum, count, rgba, value, depth);
+    auto* kernel = host.domain_kind == D_CSG ? render3_kernel<true> : render3_kernel<false>;
+    kernel<<<blocks, 256, 0, st>>>(dprob, V, sum, count, rgba, value, depth);
   }
   return cudaGetLastError() == cudaSuccess ? WOS_OK : WOS_ECUDA;
 }
