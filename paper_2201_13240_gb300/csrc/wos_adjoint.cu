@@ -6,7 +6,7 @@ namespace wos {
 size_t adjoint_smem(const AdjLaunch& L, int real_bytes) {
   size_t smem = (size_t)L.problem_bytes;
   if (L.pass == 2 && L.mode != ADJ_SIGMA)
-    smem += (kAdjBlock / 32) * (real_bytes == 8 ? sizeof(AdjStage<double>) : sizeof(AdjStage<float>)) +
+    smem += (kAdjBlock / 32) * 4 * (size_t)L.dim * 33 * (real_bytes == 8 ? sizeof(AdjTap<double>) : sizeof(AdjTap<float>)) +
             (size_t)L.priv_nodes * (size_t)real_bytes;
   return smem;
 }

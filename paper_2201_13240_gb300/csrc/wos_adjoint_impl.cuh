@@ -86,15 +86,15 @@ struct alignas(16) AdjTap {
   R b, c;
   int off;
 };
-template <typename R>
+template <int DIM, typename R>
 struct AdjStage {
-  AdjTap<R> tap[12 * 33];
+  AdjTap<R> tap[4 * DIM * 33];
 };
 
 // Add vN N_m + vG . grad N_m + vL Lap N_m at y to grad[m] over the 4^DIM nodes of the cubic
 // B-spline support (indices clamped as in grid_bspline), for every lane of the warp that wants
 // it; all lanes call.  grad is indexed j0 + s1 j1 + s2 j2: the grid's own layout in global memory, or
-// the per-CTA copy's (adj_strides).
+// the per-CTA copy's (adjoint_copy).
 //
 // With B, B', B'' the basis and its derivatives along an axis, the tap of controls (i, j, k) is
 //   Bz (X By + Bx Y) + Z Bx By,   X = vN Bx + vG_x Bx' + vL Bx'',  Y, Z likewise without vN,
@@ -109,7 +109,7 @@ struct AdjStage {
 // kernels 21.8 -> 18.9 ms).  Without the atomics 12.3 ms.
 template <int DIM, typename R, typename A>
 __device__ void bspline_scatter(const DevField<R>& F, const R* y, bool want, R vN, const R* vG, R vL, A* grad,
-                                int64_t s1, int64_t s2, AdjStage<R>* st) {
+                                int64_t s1, int64_t s2, AdjStage<DIM, R>* st) {
   unsigned todo = __ballot_sync(0xffffffffu, want);
   if (todo == 0u) return;
   const int lane = threadIdx.x & 31;
@@ -213,14 +213,13 @@ __global__ void __launch_bounds__(kAdjBlock, 4) WOS_ADJOINT_KERNEL(AdjLaunch L) 
   }
   // alpha: each warp's staged scatters, and the CTA's accumulators in the walk's precision (FP32
   // shared atomics are native)
-  AdjStage<R>* stage = reinterpret_cast<AdjStage<R>*>(smem_raw + L.problem_bytes) + (threadIdx.x >> 5);
-  R* gpriv = reinterpret_cast<R*>(smem_raw + L.problem_bytes + (kAdjBlock / 32) * sizeof(AdjStage<R>));
+  AdjStage<DIM, R>* stage = reinterpret_cast<AdjStage<DIM, R>*>(smem_raw + L.problem_bytes) + (threadIdx.x >> 5);
+  R* gpriv = reinterpret_cast<R*>(smem_raw + L.problem_bytes + (kAdjBlock / 32) * sizeof(AdjStage<DIM, R>));
   const bool priv = ALPHA && L.priv_nodes > 0;
   R* totals = reinterpret_cast<R*>(L.totals);
   const DevProblem<R>& Pg0 = *reinterpret_cast<const DevProblem<R>*>(L.problem);
   const int64_t ares0 = Pg0.alpha.res[0], ares1 = Pg0.alpha.res[1];
-  int64_t ps1 = 0, ps2 = 0;
-  adj_strides(ares0, ares1, &ps1, &ps2);
+  const int64_t ps1 = L.priv_s1, ps2 = L.priv_s2;
   if (priv)
     for (int i = threadIdx.x; i < L.priv_nodes; i += blockDim.x) gpriv[i] = R(0);
   __syncthreads();

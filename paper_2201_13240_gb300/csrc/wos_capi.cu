@@ -1337,16 +1337,13 @@ int adjoint_gradients(wos_ctx* ctx, const wos_problem* pr, const float* pts, int
   L.stats = reinterpret_cast<unsigned long long*>(stats);
   L.radial_tab = ctx->radial_tab[pr->dim - 2];
   if (grad_alpha) {
-    // grids of up to 8192 nodes are accumulated per CTA in shared memory, where the padded copy fits
-    const int64_t planes = pr->dim == 3 ? H.alpha.res[2] : 1;
-    int64_t s1 = 0, s2 = 0;
-    wos::adj_strides(H.alpha.res[0], H.alpha.res[1], &s1, &s2);
-    if ((int64_t)H.alpha.res[0] * H.alpha.res[1] * planes <= 8192) {
-      L.priv_nodes = (int)(s2 * planes);
-      L.pass = 2;
-      L.problem_bytes = (int)(fp64 ? sizeof(DevProblem<double>) : sizeof(DevProblem<float>));
-      if (wos::adjoint_smem(L, fp64 ? 8 : 4) > 200 * 1024) L.priv_nodes = 0;
-    }
+    L.pass = 2;
+    L.problem_bytes = (int)(fp64 ? sizeof(DevProblem<double>) : sizeof(DevProblem<float>));
+    const wos::AdjointCopy copy = wos::adjoint_copy(pr->dim, H.alpha.res[0], H.alpha.res[1], H.alpha.res[2],
+                                                    (int64_t)wos::adjoint_smem(L, fp64 ? 8 : 4), fp64 ? 8 : 4);
+    L.priv_nodes = copy.nodes;
+    L.priv_s1 = copy.s1;
+    L.priv_s2 = copy.s2;
   }
   return adjoint_run(ctx, pr, L, fp64, st);
 }

@@ -303,6 +303,14 @@ int wos_hc_nf_blocks(int dim, int mesh, int series, int bspline, uint64_t walks)
   return wos::nf_blocks(dim, mesh != 0, series != 0, bspline != 0, walks);
 }
 int wos_hc_gradient_form(int compiled, int bspline) { return wos::gradient_form(compiled != 0, bspline != 0); }
+// out: row stride, plane stride, nodes, resident blocks per SM
+void wos_hc_adjoint_copy(int dim, const int64_t* res, int64_t other, int real_bytes, int* out) {
+  const wos::AdjointCopy c = wos::adjoint_copy(dim, res[0], res[1], res[2], other, real_bytes);
+  out[0] = c.s1;
+  out[1] = c.s2;
+  out[2] = c.nodes;
+  out[3] = wos::adjoint_blocks(other + (int64_t)c.nodes * real_bytes);
+}
 int wos_hc_finds_item_again(int gathers, int lanes) { return wos::finds_item_again(gathers != 0, lanes); }
 
 // FP32 uniforms of the walk kernels from Philox words

@@ -80,17 +80,6 @@ struct WalkLaunch {
 };
 
 enum { ADJ_SIGMA = 0, ADJ_ALPHA = 1 };
-// The per-CTA copy of an alpha grid in shared memory: strides of its rows and planes.  The 32 taps a
-// warp adds at once are 4 x 4 x 2 neighbours; with a row stride of 4 (mod 8) and a plane stride of
-// 16 (mod 32) they lie in 32 different banks.
-#if defined(__CUDACC__)
-__host__ __device__
-#endif
-inline void adj_strides(int64_t res0, int64_t res1, int64_t* s1, int64_t* s2) {
-  *s1 = res0 + (12 - res0 % 8) % 8;
-  const int64_t plane = *s1 * res1;
-  *s2 = plane + (48 - plane % 32) % 32;
-}
 
 // adjoint launch: d(sum_p grad_u[p] mean_u[p]) / d(sigma grid nodes), added to grad_sigma
 struct AdjLaunch {
@@ -112,6 +101,7 @@ struct AdjLaunch {
   double* grad_alpha;             // [alpha grid nodes], accumulated (alpha launches)
   int mode;                       // ADJ_SIGMA, or ADJ_ALPHA (with sigma's gradient too if grad_sigma is set)
   int priv_nodes;                 // > 0: accumulate per CTA in shared memory over this many nodes
+  int priv_s1, priv_s2;           // row and plane strides of that copy (adjoint_copy)
   unsigned long long* stats;      // optional
   unsigned long long* work_counter;
   const float* radial_tab;

@@ -86,4 +86,31 @@ WOS_RULE int nf_blocks(int dim, bool mesh, bool series, bool bspline, uint64_t w
 // 5,003 239 / 222, 10,000 270 / 263, 16,384 325 / 327, 30,000 380 / 403, 65,536 522 / 599.
 WOS_RULE bool host_staged(int64_t npts) { return npts <= 12288; }
 
+// The per-CTA copy of an alpha grid in shared memory that an adjoint launch adds up in: strides of its rows
+// and planes, and its size (nodes 0: no copy, the gradients go to global memory; grids above 8192 nodes).
+struct AdjointCopy {
+  int s1, s2, nodes;
+};
+// resident blocks per SM of an adjoint kernel with so many bytes of shared memory; its registers allow four
+WOS_RULE int adjoint_blocks(int64_t bytes) {
+  if (bytes > 200 * 1024) return 0;
+  const int64_t n = 228 * 1024 / (bytes + 1024);  // an SM's shared memory, with what the system keeps of it
+  return n < 4 ? (int)n : 4;
+}
+// `other`: the block's further bytes (problem, staged scatters).  The 32 taps that a warp adds at once are 4 x 4 x
+// 2 neighbours: with a row stride of 4 (mod 8) and in 3D a plane stride of 16 (mod 32) they lie in 32
+// different banks (16^3 controls 17.3 -> 14.2 ms together with the warp-wide scatter).  Where the padding
+// for that costs a resident block, rows and planes are padded by one, which keeps the worst strides away.
+WOS_RULE AdjointCopy adjoint_copy(int dim, int64_t res0, int64_t res1, int64_t res2, int64_t other, int real_bytes) {
+  const int64_t planes = dim == 3 ? res2 : 1;
+  if (res0 * res1 * planes > 8192) return AdjointCopy{0, 0, 0};
+  const int64_t p1 = res0 + (12 - res0 % 8) % 8, rows = p1 * res1;
+  const int64_t p2 = dim == 3 ? rows + (48 - rows % 32) % 32 : rows;
+  const int64_t c1 = res0 + 1, c2 = c1 * res1 + 1;
+  const int padded = adjoint_blocks(other + p2 * planes * real_bytes);
+  const int close = adjoint_blocks(other + c2 * planes * real_bytes);
+  if (padded > 0 && padded >= close) return AdjointCopy{(int)p1, (int)p2, (int)(p2 * planes)};
+  return close > 0 ? AdjointCopy{(int)c1, (int)c2, (int)(c2 * planes)} : AdjointCopy{0, 0, 0};
+}
+
 }  // namespace wos

@@ -63,3 +63,26 @@ def test_gradient_forms(hc):
     fields name the same one."""
     assert hc.wos_hc_gradient_form(1, 0) == 2
     assert hc.wos_hc_gradient_form(0, 0) == hc.wos_hc_gradient_form(0, 1) == hc.wos_hc_gradient_form(1, 1) == 1
+
+
+@pytest.mark.parametrize("real", [4, 8])
+@pytest.mark.parametrize("res", [(4, 4, 4), (8, 8, 8), (16, 16, 16), (16, 16, 32), (5, 5, 327), (4, 4, 512), (20, 20, 20),
+                                 (17, 16, 32), (64, 128, 1), (65, 126, 1), (4, 2048, 1), (8192, 1, 1), (1, 1, 8192), (65, 127, 1)])
+def test_adjoint_copies_fit_and_cost_no_block(hc, res, real):
+    """The padded copy of an alpha grid holds every node at its own address, and costs no resident block
+    against rows and planes that are one apart; grids above 8192 nodes have none."""
+    dim, other = (2 if res[2] == 1 else 3), 5312 + 4 * 33 * 4 * 4 * (2 if res[2] == 1 else 3) * real
+    r, out = (C.c_int64 * 3)(*res), (C.c_int * 4)()
+    hc.wos_hc_adjoint_copy.argtypes = [C.c_int, C.POINTER(C.c_int64), C.c_int64, C.c_int, C.POINTER(C.c_int)]
+    hc.wos_hc_adjoint_copy(dim, r, other, real, out)
+    s1, s2, nodes, blocks = out
+    close = ((res[0] + 1) * res[1] + 1) * res[2] * real + other
+    want = 0 if close > 200 * 1024 else min(4, 228 * 1024 // (close + 1024))
+    if res[0] * res[1] * res[2] > 8192:
+        assert nodes == 0
+    elif nodes:
+        assert s1 >= res[0] and (dim == 2 or s2 >= s1 * (res[1] - 1) + res[0])
+        assert (res[0] - 1) + s1 * (res[1] - 1) + s2 * (res[2] - 1) < nodes
+        assert blocks >= want and other + nodes * real <= 200 * 1024
+    else:
+        assert want == 0
