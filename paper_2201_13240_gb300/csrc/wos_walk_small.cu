@@ -22,11 +22,13 @@ struct SumRun {
 // 2048 warps of the ~3000 that fit and lasted four walks and the longest one's tail.  Measured:
 // 3,000 points x 64 walks on a mesh 476 -> 266 ms, 32^2 x 256 of the 2D square 494 -> 461 us.
 //
-// The order of the sums is the persistent kernel's: FP32 partial sums per lane, shifted by the
-// lane's first walk of the point, over the walks that lane would have run had one warp taken
-// 128 consecutive walks, each lane that is free claiming the next one (lanes free at the same
-// iteration in lane order, GATHERED: once four lanes are free).  A solve's sums therefore
-// do not depend on which warp ran which walk, and equal those of larger chunks' launches.
+// The sums are FP32 partial sums per lane, shifted by the lane's first walk of the point, over the walks
+// that lane would have run had one warp taken 128 consecutive walks, each lane that is free claiming
+// the next one (lanes free at the same iteration in lane order, GATHERED: once four lanes are free).
+// So they do not depend on which warp ran which walk, and they are the sums that small solves had
+// when the walk kernels formed them.  Larger solves add in other orders, and kernels compiled for 2D or
+// B-spline problems, and batches of such, in FP64 (sums_in_fp64): on the two sides of kSpreadItems walks
+// those problems' sums differ by the rounding of FP32 partial sums.
 template <bool GATHERED>
 __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__ acc, const uint32_t* __restrict__ iters,
                                                        const uint32_t* __restrict__ point,
@@ -34,7 +36,7 @@ __global__ void __launch_bounds__(128) walk_sum_kernel(const float* __restrict__
                                                        const int64_t* walk_end, int64_t npts, double* sum,
                                                        double* sumsq, unsigned long long* count) {
   if (walk_end != nullptr) all = (uint64_t)__ldg(&walk_end[npts - 1]);  // per-point walk counts
-  if (all > kSpreadItems) return;  // the walk kernel added these up itself
+  if (all > kSpreadItems) return;  // the walk kernel, or the other of two launches, added these up itself
   const uint32_t total = (uint32_t)all;
   const uint32_t lane = threadIdx.x & 31, base = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kChunkMin;
   if (base >= total) return;
