@@ -21,7 +21,7 @@ BUILD_DIR = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libwos.so")
 HOSTCHECK = os.path.join(HERE, "libwos_hostcheck.so")
 
-CU_SOURCES = ["wos_capi.cu", "wos_walk_f32.cu", "wos_walk_small.cu", "wos_walk_counts.cu", "wos_walk_f64.cu",
+CU_SOURCES = ["wos_capi.cu", "wos_walk_f32.cu", "wos_walk_small.cu", "wos_walk_f64.cu",
               "wos_nf_f32.cu", "wos_nf_f64.cu", "wos_adjoint.cu", "wos_render.cu", "wos_jit.cu", "wos_mesh.cpp", "wos_handles.cu", "wos_peaks.cu"]
 HEADERS = ["wos_math.cuh", "wos_problem.cuh", "wos_walk_impl.cuh", "wos_nf_impl.cuh", "wos_adjoint_impl.cuh",
            "wos_internal.h", "wos_rules.h", "wos_mesh.h", "wos_jit.h", "wos_capi_state.h"]

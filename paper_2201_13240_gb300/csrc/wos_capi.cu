@@ -422,6 +422,7 @@ bool has_bspline(const DevProblem<double>& P) {
 // returns at once.  bspline: of a problem's fields; batches choose their register cap by a schedule.
 cudaError_t launch_generic_f32(wos::WalkLaunch L, int num_sms, bool bspline, cudaStream_t st) {
   const bool batch = L.probs != nullptr;
+  if (L.ww_lo != 0.0) return wos::launch_walks_small_f32(L, num_sms, st);  // windows have the one form
   if (L.item_acc != nullptr) {
     if (!batch) L.regs_variant = wos::value_variant(L.dim, bspline, wos::walks_of_launch(L.total_items, true));
     const cudaError_t e = (batch || L.walk_end != nullptr) ? wos::launch_walks_counts_f32(L, num_sms, st)

@@ -121,7 +121,7 @@ cudaError_t launch_adjoint_kernel(const AdjLaunch& L, cudaKernel_t kernel, int r
 
 // launch the persistent walk kernel; returns a cudaError_t
 cudaError_t launch_walks_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream);
-// small solves' forms (SpreadForm): equal counts; per-point counts and batches
+// small solves' forms (SpreadForm): equal counts, and windows of any size; per-point counts and batches
 cudaError_t launch_walks_small_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream);
 cudaError_t launch_walks_counts_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream);
 cudaError_t launch_walks_f64(const WalkLaunch& L, int num_sms, cudaStream_t stream);

@@ -43,10 +43,11 @@ WOS_RULE int gradient_form(bool compiled, bool bspline) { return compiled && !bs
 // number of walks in the launch.  As a choice at a walk's end it costs large solves up to 5 % (2D B-spline
 // annulus, 4.2e6 walks, 4.30 -> 4.51 ms; noise cube at five blocks 8.94 -> 9.05 ms), so of the generic kernels
 // large solves run the first form (4.35 ms).  Small solves with per-point counts, and small batches, run the
-// second: 3 to 11 % faster than the third.  Small solves of equal counts keep the third: they wait for a lone
-// walk's steps, and those are the faster in it (4096 x 256 windows 18.8 ms against 21.3, the 2D square's 32^2 x
-// 256 walks 475 us against 530; 20.6 ms and 522 us in one module with the batches' kernels).  Compiled kernels hold the choice: a second kernel would add half to their compilation (0.1 to
-// 0.8 s), and it costs nothing but in 3D windows (1.20 -> 1.22 ms).
+// second: 2 to 11 % faster than the third.  Small solves of equal counts keep the third: they wait for a lone
+// walk's steps, and those are the faster in it (4096 x 256 windows 20.6 ms against 21.3, the 2D square's 32^2 x
+// 256 walks 522 us against 530).  Windows wait for their longest walk at any size, and have that form alone
+// (1.1e6 walks 18.5 ms against 18.7).  Compiled kernels hold the choice: a second kernel would add half to
+// their compilation (0.1 to 0.8 s), and it costs nothing but in 3D windows (1.20 -> 1.22 ms).
 enum SpreadForm { SPREAD_NEVER = 0, SPREAD_ALWAYS = 1, SPREAD_BY_SIZE = 2 };
 
 // The register cap of the generic FP32 value kernel for a launch of `walks` walks: variant 0, five blocks

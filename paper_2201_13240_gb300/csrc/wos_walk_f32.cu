@@ -1,4 +1,7 @@
-// wos_walk_f32.cu -- FP32 walk kernels (2D and 3D): the production path.
+// wos_walk_f32.cu -- FP32 walk kernels (2D and 3D): the production path.  All forms of the generic kernels
+// (SpreadForm) are compiled here together: the compiler shapes field_eval, which they call, by all of its
+// callers in a file, and in files apart 2D B-spline fields were rounded differently (sums 5e-8 off; the
+// tests compare the forms bit by bit).
 #include "wos_walk_impl.cuh"
 
 namespace wos {
@@ -6,6 +9,16 @@ namespace wos {
 cudaError_t launch_walks_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
   return (L.dim == 2) ? launch_walks_t<2, float>(L, num_sms, stream)
                       : launch_walks_t<3, float>(L, num_sms, stream);
+}
+
+cudaError_t launch_walks_small_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
+  return (L.dim == 2) ? launch_walks_t<2, float, SPREAD_BY_SIZE>(L, num_sms, stream)
+                      : launch_walks_t<3, float, SPREAD_BY_SIZE>(L, num_sms, stream);
+}
+
+cudaError_t launch_walks_counts_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
+  return (L.dim == 2) ? launch_walks_t<2, float, SPREAD_ALWAYS>(L, num_sms, stream)
+                      : launch_walks_t<3, float, SPREAD_ALWAYS>(L, num_sms, stream);
 }
 
 cudaError_t launch_walks_kernel(const WalkLaunch& L, cudaKernel_t kernel, int real_bytes, int num_sms,

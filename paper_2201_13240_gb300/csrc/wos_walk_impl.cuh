@@ -814,12 +814,15 @@ cudaError_t launch_walks_t(const WalkLaunch& L, int num_sms, cudaStream_t stream
       return launch_walks_m<DIM, R, false, false, false, true>(L, num_sms, stream);
     }
   }
-  const bool ww = L.ww_lo > 0.0;
+  if constexpr (SPREAD == SPREAD_BY_SIZE || sizeof(R) == 8) {  // the one form of FP32 windows
+    if (L.ww_lo > 0.0) {
+      if constexpr (DIM == 3)
+        if (L.mesh) return launch_walks_m<DIM, R, true, false, true, false, false, 0, SPREAD>(L, num_sms, stream);
+      return launch_walks_m<DIM, R, false, false, true, false, false, 0, SPREAD>(L, num_sms, stream);
+    }
+  }
   if constexpr (DIM == 3)
-    if (L.mesh)
-      return ww ? launch_walks_m<DIM, R, true, false, true, false, false, 0, SPREAD>(L, num_sms, stream)
-                : launch_walks_m<DIM, R, true, false, false, false, false, 0, SPREAD>(L, num_sms, stream);
-  if (ww) return launch_walks_m<DIM, R, false, false, true, false, false, 0, SPREAD>(L, num_sms, stream);
+    if (L.mesh) return launch_walks_m<DIM, R, true, false, false, false, false, 0, SPREAD>(L, num_sms, stream);
   if constexpr (sizeof(R) == 4) {  // value_variant
     if constexpr (SPREAD == SPREAD_NEVER)
       if (L.regs_variant == 1) return launch_walks_m<DIM, R, false, false, false, false, false, 8>(L, num_sms, stream);

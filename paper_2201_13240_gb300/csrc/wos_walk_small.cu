@@ -1,13 +1,7 @@
-// wos_walk_small.cu -- small FP32 solves of equal counts: the generic walk kernels that may run one walk per
-// lane and leave the sums to walk_sum_kernel, and that kernel.
+// wos_walk_small.cu -- the sums of small FP32 solves, whose walk kernels run one walk per lane.
 #include "wos_walk_impl.cuh"
 
 namespace wos {
-
-cudaError_t launch_walks_small_f32(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
-  return (L.dim == 2) ? launch_walks_t<2, float, SPREAD_BY_SIZE>(L, num_sms, stream)
-                      : launch_walks_t<3, float, SPREAD_BY_SIZE>(L, num_sms, stream);
-}
 
 struct SumRun {
   uint32_t p, n;        // point, walks

@@ -21,7 +21,8 @@ def _counts(npts, total, rng):
 
 @pytest.mark.parametrize("total", [1, 900, LIMIT, LIMIT + 1])
 @pytest.mark.parametrize("kind,spec", [("square2d", True), ("noise_annulus", True), ("noise_cube", True),
-                                       ("hifreq", True), ("square2d", False), ("noise_cube", False)])
+                                       ("hifreq", True), ("square2d", False), ("noise_cube", False),
+                                       ("hifreq", False)])
 def test_per_point_counts_sum_the_walks(kind, spec, total):
     """A lane adds n consecutive walks of a point in FP32, at most all of them: the rounding is at most
     n * 2^-24 of the sum of magnitudes, and for the squares (shifted by a walk's value) 8 n * 2^-24 of
@@ -86,3 +87,28 @@ def test_batches_sum_the_same_walks_on_either_path(spec, per_point):
     rms = (r2 * m).sqrt()  # at least the sum of magnitudes
     assert torch.all((s - r).abs() <= tol * rms)
     assert torch.all((s2 - r2).abs() <= 8 * tol * r2 * m)
+
+
+@pytest.mark.parametrize("kind", ["square2d", "cube3d", "noise_annulus", "noise_cube", "hifreq"])
+def test_forms_of_the_generic_kernel_round_alike(kind):
+    """One walk per point: its sum is its estimate, a product of two FP32 numbers and so exact in FP64, in the
+    form that writes estimates, in the small solves' form and in the form of per-point counts."""
+    import torch
+
+    import paper_2201_13240_gb300 as wos
+    ctx = wos.Context(0)
+    desc = {"square2d": W.square2d_problem, "cube3d": W.cube3d_problem, "noise_annulus": W.noise_annulus_problem,
+            "noise_cube": W.noise_cube_problem, "hifreq": W.hifreq_alpha_problem}[kind]()
+    prob = ctx.problem(desc)
+    sb = ctx.sigma_bar(prob, 32)[0]
+    n, rng = 3000, np.random.default_rng(2)
+    r, t = np.sqrt(rng.uniform(0.4 ** 2, 1.05 ** 2, n)), rng.uniform(0, 2 * np.pi, n)
+    pts = np.stack([r * np.cos(t), r * np.sin(t)]).astype(np.float32) if kind == "noise_annulus" else \
+        W.uniform_in_box(desc["dim"], n, 0.02, 0.98, 5)
+    pts, ones = torch.from_numpy(pts).cuda(), torch.ones(n, dtype=torch.int32, device="cuda")
+    for window in (None, (0.5, 1.5)):
+        u = ctx.walk_estimates(prob, pts, 1, 1e-3, sb, seed=9, window=window)[0][:, 0]
+        for walks in (1, ones):
+            (s, s2, _), _ = ctx.solve(prob, pts, walks, 1e-3, sb, seed=9, window=window)
+            assert torch.equal(s, u)
+            assert torch.allclose(s2, u * u, rtol=1e-15, atol=0)
