@@ -437,7 +437,7 @@ cudaError_t launch_generic_f32(wos::WalkLaunch L, int num_sms, bool bspline, cud
 // and decides, one for few walks and one for many.
 cudaError_t launch_nf_sized(wos::WalkLaunch L, int num_sms, bool bspline, cudaStream_t st) {
   auto blocks = [&](uint64_t walks) { return wos::nf_blocks(L.dim, L.mesh != 0, L.nf_series > 0, bspline, walks); };
-  const uint64_t few = wos::nf_few_walks(bspline);
+  const uint64_t few = wos::nf_few_walks(L.mesh != 0, bspline);
   if (L.walk_end != nullptr && blocks(few) != blocks(L.total_items)) {
     L.regs_variant = blocks(few);
     L.nf_at_most = few;

@@ -399,9 +399,14 @@ template <int DIM, typename R>
 cudaError_t launch_nf_t(const WalkLaunch& L, int num_sms, cudaStream_t stream) {
   const bool series = L.nf_series > 0;
   if constexpr (DIM == 3)
-    if (L.mesh)
+    if (L.mesh) {
+      if constexpr (sizeof(R) == 4)
+        if (L.regs_variant == 5)
+          return series ? launch_nf_m<DIM, R, true, true, 5>(L, num_sms, stream)
+                        : launch_nf_m<DIM, R, true, false, 5>(L, num_sms, stream);
       return series ? launch_nf_m<DIM, R, true, true, 4>(L, num_sms, stream)
                     : launch_nf_m<DIM, R, true, false, 4>(L, num_sms, stream);
+    }
   if constexpr (sizeof(R) == 4) {
     if (series && L.regs_variant == 5) return launch_nf_m<DIM, R, false, true, 5>(L, num_sms, stream);
     if (!series && L.regs_variant == 6) return launch_nf_m<DIM, R, false, false, 6>(L, num_sms, stream);

@@ -72,12 +72,15 @@ WOS_RULE uint64_t walks_of_launch(uint64_t total, bool small_launch) {
 // 3.53 / 3.89, 3.9e5 walks 2.79 / 2.78 / 2.44 and 4.57 / 4.49 / 4.30 (six blocks round the series otherwise: other
 // walks), 2.1e6 walks 8.57 / 8.33 / 7.68 and 14.8 / 14.3 / 14.7.  Noise cube (B-spline fields), 0 and 8 terms: 2.0e5
 // walks 2.74 / 3.54 / 4.11 and 5.77 / 6.61 / 7.13, 2.1e6 walks 13.1 / 14.3 / 15.8 and 28.1 / 27.1 / 27.6; in
-// 2D (annulus, 0 terms) 0.94 / 0.99 / 1.17 and 4.21 / 4.02 / 4.06.  Mesh, 1.1e6 walks: 54.7 / 55.2 / 59.6 and 68.4 / 69.4 /
-// 72.0.  nf_few_walks: the most walks that count as few.
-WOS_RULE uint64_t nf_few_walks(bool bspline) { return bspline ? 1ull << 20 : 1ull << 18; }
+// 2D (annulus, 0 terms) 0.94 / 0.99 / 1.17 and 4.21 / 4.02 / 4.06.  Mesh, 20,480 triangles, 4 / 5:
+// 1.3e5 walks 20.7 / 23.1 and 23.8 / 25.7, 5.2e5 walks 38.9 / 40.7 and 43.9 / 48.2, 1.05e6 walks 68.0 / 65.2 and 76.9 /
+// 75.0, 4.2e6 walks 240 / 225 and 270 / 260.  nf_few_walks: the most walks that count as few.
+WOS_RULE uint64_t nf_few_walks(bool mesh, bool bspline) {
+  return mesh ? 3ull << 18 : (bspline ? 1ull << 20 : 1ull << 18);
+}
 WOS_RULE int nf_blocks(int dim, bool mesh, bool series, bool bspline, uint64_t walks) {
-  if (mesh || walks <= nf_few_walks(bspline)) return 4;
-  if (series) return 5;
+  if (walks <= nf_few_walks(mesh, bspline)) return 4;
+  if (mesh || series) return 5;
   return bspline && dim == 3 ? 4 : 6;
 }
 

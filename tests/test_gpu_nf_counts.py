@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("terms", [0, 8])
-@pytest.mark.parametrize("kind,few", [("square2d", 1 << 18), ("cube3d", 1 << 18), ("noise_cube", 1 << 20)])
+@pytest.mark.parametrize("kind,few", [("square2d", 1 << 18), ("cube3d", 1 << 18), ("noise_cube", 1 << 20), ("mesh", 3 << 18)])
 @pytest.mark.parametrize("over", [None, 0, 1])
 def test_sums_equal_the_walks(kind, few, terms, over):
     """over: walks above the limit (None: a handful).  Estimates are added in FP64: the sums agree with the
@@ -19,7 +19,8 @@ def test_sums_equal_the_walks(kind, few, terms, over):
 
     import paper_2201_13240_gb300 as wos
     ctx = wos.Context(0)
-    desc = {"square2d": W.square2d_problem, "cube3d": W.cube3d_problem, "noise_cube": W.noise_cube_problem}[kind]()
+    desc = {"square2d": W.square2d_problem, "cube3d": W.cube3d_problem, "noise_cube": W.noise_cube_problem,
+            "mesh": lambda: W.mesh_manufactured_problem(level=2, tol=0.25)}[kind]()
     prob = ctx.problem(desc)
     sb = ctx.sigma_bar(prob, 32)[0]
     npts, rng = 2048, np.random.default_rng(7)
@@ -28,7 +29,8 @@ def test_sums_equal_the_walks(kind, few, terms, over):
     counts[1] += counts[5]
     counts[5] = 0
     most = int(counts.max())
-    pts = torch.from_numpy(W.uniform_in_box(desc["dim"], npts, 0.02, 0.98, 5)).cuda()
+    pts = W.mesh_interior_points(npts, 5) if kind == "mesh" else W.uniform_in_box(desc["dim"], npts, 0.02, 0.98, 5)
+    pts = torch.from_numpy(pts).cuda()
     (s, s2, n), st = ctx.solve_nf(prob, pts, torch.from_numpy(counts).cuda(), 1e-3, sb, seed=7, series_terms=terms)
     u, _, _ = ctx.walk_estimates_nf(prob, pts, most, 1e-3, sb, seed=7, series_terms=terms)
     assert np.array_equal(n.cpu().numpy(), counts) and int(st[1]) == total

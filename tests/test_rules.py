@@ -43,12 +43,15 @@ def test_register_variants_by_the_walks_of_a_launch(hc):
 
 
 def test_next_flight_register_caps(hc):
-    """More than four blocks per SM only where they are the faster ones: never on meshes or for few walks, and
-    never for the printed approximations with 3D B-spline fields, whose taps would spill."""
+    """More than four blocks per SM only where they are the faster ones: never for few walks (more of them
+    count as few on meshes and with B-spline fields), and never for the printed approximations with 3D
+    B-spline fields, whose taps would spill."""
     hc.wos_hc_nf_blocks.argtypes = [C.c_int] * 4 + [C.c_uint64]
     for series in (0, 1):
-        for walks in (1, 1 << 18, 1 << 20, 1 << 30):
-            assert hc.wos_hc_nf_blocks(3, 1, series, 0, walks) == 4
+        for bspline in (0, 1):
+            for walks in (1, 1 << 18, 3 << 18):
+                assert hc.wos_hc_nf_blocks(3, 1, series, bspline, walks) == 4
+            assert hc.wos_hc_nf_blocks(3, 1, series, bspline, (3 << 18) + 1) == 5
         for dim in (2, 3):
             assert hc.wos_hc_nf_blocks(dim, 0, series, 0, 1 << 18) == 4
             assert hc.wos_hc_nf_blocks(dim, 0, series, 1, 1 << 20) == 4
