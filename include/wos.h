@@ -433,7 +433,9 @@ int wos_batch_get_schedule(const wos_batch* batch, wos_schedule* sched);
    chunk rule and chunks 64..2048, at both register caps), each with walks per point
    reduced to max(1, walks >> trial_shift) (0..16; 4 is a sixteenth), keeps the fastest in the
    batch and returns it with its trial time (*best_ms) and the default schedule's
-   (*default_ms; either pointer may be NULL).  It allocates trial accumulators on the device,
+   (*default_ms; either pointer may be NULL).  Trials run as the launch that they stand for
+   would, summed afterwards at most 2^20 walks and in the kernel above; those of small launches
+   are repeated, each candidate's best counting.  It allocates trial accumulators on the device,
    synchronises `stream` after every trial and frees them before returning: call it before
    capturing the batch's solve in a CUDA graph, not inside one.  Arguments as
    wos_solve_batch; the trial sums are discarded. */

@@ -47,7 +47,7 @@ __device__ double sd_domain(const DevProblem<double>& P, const double* x) {
 // evaluated the plane and every primitive in FP64, some 25 operations each with a square root.  The
 // FP32 pass costs a fraction of that; where its intervals do not tell the winner (a crease, a far-off
 // point) the whole list is evaluated in FP64 as before, so every step's length, and the image, is
-// the same.  Measured (1280 x 720, five primitives): 5.70 -> 2.48 ms, FP64 pipe 56 % busy; more
+// the same.  Measured (1280 x 720, five primitives): 5.70 -> 2.33 ms, FP64 instructions 74 % of their peak; more
 // resident blocks by spilling (3, 4 or 5 of 256 threads) 2.8, 2.9 and 4.3 ms.
 struct CsgF32 {
   CsgNode<float> node[kMaxCsg];
