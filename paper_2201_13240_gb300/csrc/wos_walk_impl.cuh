@@ -836,8 +836,8 @@ cudaError_t launch_walks_t(const WalkLaunch& L, int num_sms, cudaStream_t stream
 template <int DIM, typename R>
 int blocks_per_sm_t() {
   int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wos_walk_kernel<DIM, R, false, false, false, false, false, 0, SPREAD_NEVER>,
-                                                kWalkBlock, sizeof(DevProblem<R>));
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &per_sm, wos_walk_kernel<DIM, R, false, false, false, false, false, 0, SPREAD_NEVER>, kWalkBlock, sizeof(DevProblem<R>));
   return per_sm;
 }
 #endif  // !__CUDACC_RTC__
